@@ -54,7 +54,9 @@ typedef enum {
 } ddf_status;
 
 typedef enum {
-  DDF_FP32 = 0,      /* plain FP32 on CUDA cores (no TF32) */
+  DDF_FP32 = 0,      /* FP32 (no TF32): widths that are multiples of 256 on the tensor cores,
+                        each operand split exactly into three bf16 values, others on CUDA
+                        cores */
   DDF_BF16 = 1,      /* bf16 operands, FP32 accumulation on tcgen05 tensor cores */
   DDF_FP8_E4M3 = 2   /* e4m3 operands (layers 2..H), FP32 accumulation on tcgen05 */
 } ddf_precision;
@@ -512,7 +514,8 @@ ddf_status ddf_set_timeout_ns(ddf_handle h, uint64_t ns);
 
 /* Rays per internal chunk of a query (default 1,048,576; minimum 128). Sets
  * the workspace size: about chunk * (4 W + D_in) bytes at bf16/fp8 and twice
- * that at FP32. */
+ * that at FP32 (three times, for at most 131,072 rays, where the width is a
+ * multiple of 256). */
 ddf_status ddf_set_chunk_rays(ddf_handle h, int64_t chunk);
 
 /* Tensor-core tile of the layer kernel.

@@ -116,9 +116,11 @@ void release_weight_buffers(ddf_s* h) {
   }
   for (__nv_bfloat16* q : h->wb) dev_free(h, q);
   for (__nv_bfloat16* q : h->wcal) dev_free(h, q);
+  for (__nv_bfloat16* q : h->wp) dev_free(h, q);
   for (uint8_t* q : h->wq) dev_free(h, q);
   h->wb.clear();
   h->wcal.clear();
+  h->wp.clear();
   h->wq.clear();
   dev_free(h, h->head_w);
   dev_free(h, h->head_b);
@@ -194,13 +196,13 @@ ddf_status ensure_workspace(ddf_s* h, int64_t rows) {
   const bool f32 = h->cfg.precision == DDF_FP32;
   // e4m3 activations need 1 byte, but the calibration pass of an FP8 handle
   // runs the layers in bf16 through the same buffers
-  const size_t act_elem = f32 ? 4 : 2;
-  const size_t enc_bytes = static_cast<size_t>(rows) * (f32 ? h->kp32 * 4 : h->kp16 * 2);
+  const bool planes = f32 && h->f32_clusters > 0;  // three bf16 planes of one pass's rows
+  const size_t elem = planes ? 6 : f32 ? 4 : 2;
+  const size_t r = static_cast<size_t>(planes ? std::min(rows, h->f32_pass) : rows);
   ddf_status st;
-  if ((st = dev_alloc(h, &h->ws_enc, enc_bytes)) != DDF_OK) return st;
+  if ((st = dev_alloc(h, &h->ws_enc, r * (f32 ? h->kp32 : h->kp16) * elem)) != DDF_OK) return st;
   for (int i = 0; i < 2; ++i)
-    if ((st = dev_alloc(h, &h->ws_act[i], static_cast<size_t>(rows) * W * act_elem)) != DDF_OK)
-      return st;
+    if ((st = dev_alloc(h, &h->ws_act[i], r * W * elem)) != DDF_OK) return st;
   if (!f32) {
     void* p;
     if ((st = dev_alloc(h, &p, static_cast<size_t>(rows) * max_partials(W) * sizeof(float2))) != DDF_OK)
@@ -257,8 +259,55 @@ ddf::HeadOut shift_out(ddf::HeadOut o, int64_t off) {
   return o;
 }
 
+// One pass of an FP32 query on the tensor cores: the encoding and every
+// activation as three bf16 planes (tc_gemm_f32.cu), FP32 rows for the head.
+ddf_status forward_f32_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  {
+    ProfScope ps(h, kProfEncode, st);
+    DDF_CK(ddf::launch_encode_planes(rays, m, h->cfg.octaves, h->kp32,
+                                     static_cast<__nv_bfloat16*>(h->ws_enc), st));
+  }
+  const int64_t tiles = ((m + 255) / 256) * static_cast<int64_t>(W / 256);
+  const int clusters = static_cast<int>(std::min<int64_t>(tiles, h->f32_clusters));
+  for (int l = 0; l < H; ++l) {
+    const void* a_base = l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1];
+    ddf::TcF32Params p{};
+    p.M = m;
+    p.N = W;
+    p.K = l == 0 ? h->kp32 : W;
+    p.bias = h->bias[l];
+    if (l == H - 1)
+      p.out_f32 = static_cast<float*>(h->ws_act[l & 1]);
+    else
+      p.out_planes = static_cast<__nv_bfloat16*>(h->ws_act[l & 1]);
+    p.status = h->status_dev;
+    p.timeout_ns = h->timeout_ns;
+    CUtensorMap tmA;
+    if (!make_tmap(&tmA, a_base, false, p.K, 3 * static_cast<uint64_t>(m),
+                   static_cast<uint64_t>(p.K) * 2, 128))
+      return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
+    ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
+    DDF_CK(ddf::launch_tc_gemm_f32(tmA, h->tmB[l], p, clusters, st));
+  }
+  ProfScope ps(h, kProfHead, st);
+  DDF_CK(ddf::launch_head_f32(static_cast<const float*>(h->ws_act[(H - 1) & 1]), m, W, h->head_w,
+                              h->head_b, out, st));
+  return DDF_OK;
+}
+
 ddf_status forward_f32(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
   const int W = h->cfg.width;
+  if (h->f32_clusters > 0) {
+    for (int64_t off = 0; off < m; off += h->f32_pass) {
+      const ddf_status s =
+          forward_f32_tc(h, shift_rays(rays, off),
+                         static_cast<int>(std::min<int64_t>(h->f32_pass, m - off)),
+                         shift_out(out, off), st);
+      if (s != DDF_OK) return s;
+    }
+    return DDF_OK;
+  }
   {
     ProfScope ps(h, kProfEncode, st);
     DDF_CK(ddf::launch_encode_f32(rays, m, h->cfg.octaves, h->kp32, static_cast<float*>(h->ws_enc), st));
@@ -700,10 +749,10 @@ ddf_status ddf_create(const ddf_config* cfg, ddf_handle* out) {
   if (cfg->device >= ndev) return fail(DDF_ERR_INVALID_ARG, "device ordinal out of range");
   DeviceGuard g(cfg->device);
   if (!g.ok) return fail(DDF_ERR_CUDA, "cudaSetDevice failed");
+  int major = 0, minor = 0;
+  DDF_CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device));
+  DDF_CK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, cfg->device));
   if (cfg->precision != DDF_FP32) {
-    int major = 0, minor = 0;
-    DDF_CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device));
-    DDF_CK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, cfg->device));
     if (major != 10 || minor != 3)
       return fail(DDF_ERR_UNSUPPORTED, "tensor-core precisions are built for sm_103a only");
     if (get_encode_fn() == nullptr)
@@ -720,6 +769,9 @@ ddf_status ddf_create(const ddf_config* cfg, ddf_handle* out) {
   if (layered && cfg->precision != DDF_FP32 && cfg->width % 256 == 0)
     h->pair_clusters = std::min(ddf::tc_gemm_pair_max_clusters(false),
                                 ddf::tc_gemm_pair_max_clusters(true));
+  if (layered && cfg->precision == DDF_FP32 && cfg->width % 256 == 0 && major == 10 &&
+      minor == 3 && get_encode_fn() != nullptr)
+    h->f32_clusters = ddf::tc_gemm_f32_max_clusters();
   cudaError_t e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
   void* p = nullptr;
   if (e != cudaSuccess || dev_alloc(h, &p, sizeof(uint32_t)) != DDF_OK) {
@@ -789,6 +841,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     h->d_blob = static_cast<float*>(p);
     h->wf.assign(H, nullptr);
     h->bias.assign(H, nullptr);
+    h->wp.assign(H, nullptr);
     h->wb.assign(H, nullptr);
     h->wq.assign(H, nullptr);
     h->wscale.assign(H, nullptr);
@@ -802,8 +855,17 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
       h->bias[l] = static_cast<float*>(p);
       if (prec == DDF_FP32) {
         const int kp = l == 0 ? h->kp32 : W;
-        if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * kp * sizeof(float))) != DDF_OK) return s;
-        h->wf[l] = static_cast<float*>(p);
+        if (h->f32_clusters == 0) {
+          if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * kp * sizeof(float))) != DDF_OK)
+            return s;
+          h->wf[l] = static_cast<float*>(p);
+        } else {
+          if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * kp * 6)) != DDF_OK) return s;
+          h->wp[l] = static_cast<__nv_bfloat16*>(p);
+          if (!make_tmap(&h->tmB[l], h->wp[l], false, kp, 3 * static_cast<uint64_t>(W),
+                         static_cast<uint64_t>(kp) * 2, 128))
+            return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+        }
       } else if (prec == DDF_BF16 || l == 0) {
         const int kp = l == 0 ? h->kp16 : W;
         if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * kp * 2)) != DDF_OK) return s;
@@ -853,7 +915,10 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     DDF_CK(cudaMemcpy(h->bias[l], h->d_blob + off, W * sizeof(float), cudaMemcpyDeviceToDevice));
     off += W;
     if (prec == DDF_FP32) {
-      DDF_CK(ddf::launch_pack_f32(w, W, K, l == 0 ? h->kp32 : W, h->wf[l], st));
+      if (h->f32_clusters == 0)
+        DDF_CK(ddf::launch_pack_f32(w, W, K, l == 0 ? h->kp32 : W, h->wf[l], st));
+      else
+        DDF_CK(ddf::launch_pack_planes(w, W, K, l == 0 ? h->kp32 : W, h->wp[l], st));
     } else if (prec == DDF_BF16 || l == 0) {
       DDF_CK(ddf::launch_pack_bf16(w, W, K, l == 0 ? h->kp16 : W, h->wb[l], st));
       // the transposed copies of a handle that has trained (input gradients)
@@ -1499,15 +1564,25 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   DeviceGuard g(h->cfg.device);
   const int W = h->cfg.width;
   const bool f32 = h->cfg.precision == DDF_FP32;
-  const size_t act_elem = f32 ? 4 : (h->cfg.precision == DDF_BF16 ? 2 : 1);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  // FP32 on the tensor cores keeps 6 bytes a value, of as many rows at a time
+  // as fit (the same results, every row being independent of the others)
+  const bool planes = f32 && h->f32_clusters > 0;
+  int64_t rows = n;
+  if (planes) {
+    const size_t per_row = 6 * (static_cast<size_t>(h->kp32) + 2 * W);
+    rows = std::min<int64_t>(n, static_cast<int64_t>((ws_bytes - 3 * 256) / per_row));
+    if (rows > 256) rows = std::min<int64_t>(n, rows / 256 * 256);
+    if (rows < 1) return fail(DDF_ERR_INVALID_ARG, "workspace too small for this batch");
+  }
+  const size_t act_elem = planes ? 6 : f32 ? 4 : (h->cfg.precision == DDF_BF16 ? 2 : 1);
   uint8_t* p = static_cast<uint8_t*>(ws);
   void* enc = p;
-  p += up(static_cast<size_t>(n) * (f32 ? h->kp32 * 4 : h->kp16 * 2));
+  p += up(static_cast<size_t>(rows) * (f32 ? h->kp32 * (planes ? 6 : 4) : h->kp16 * 2));
   void* act0 = p;
-  p += up(static_cast<size_t>(n) * W * act_elem);
+  p += up(static_cast<size_t>(rows) * W * act_elem);
   void* act1 = p;
-  p += up(static_cast<size_t>(n) * W * act_elem);
+  p += up(static_cast<size_t>(rows) * W * act_elem);
   float2* part = f32 ? nullptr : reinterpret_cast<float2*>(p);
 
   void* save_enc = h->ws_enc;
@@ -1523,10 +1598,13 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   h->ws_rows = n;
   h->chunk = n;
   h->prof = false;
+  const int64_t save_pass = h->f32_pass;
+  if (planes) h->f32_pass = rows;
   ddf::HeadOut o{};
   o.t = out_t;
   o.vis = out_vis;
   s = run_query(h, rays, n, o, static_cast<cudaStream_t>(stream));
+  h->f32_pass = save_pass;
   h->ws_enc = save_enc;
   h->ws_act[0] = save_act0;
   h->ws_act[1] = save_act1;

@@ -45,6 +45,13 @@ struct ddf_s {
   std::vector<void*> owned;  // device allocations freed by ddf_destroy
   float* d_blob = nullptr;   // FP32 master weights
   std::vector<float*> wf;    // FP32: padded W per hidden layer
+  // FP32 on the tensor cores (width a multiple of 256): clusters of its kernel
+  // that fit the device (0: FFMA layers), the rows it takes through all layers
+  // at once (512 row blocks fill the GPU many times over, and three planes of
+  // activations, 6 bytes a value, stay small), and W as three bf16 planes
+  int f32_clusters = 0;
+  int64_t f32_pass = 131072;
+  std::vector<__nv_bfloat16*> wp;
   std::vector<float*> bias;  // per hidden layer [W]
   std::vector<__nv_bfloat16*> wb;  // bf16 W (all layers for BF16, layer 1 for FP8)
   std::vector<uint8_t*> wq;        // FP8: e4m3 codes for layers 2..H

@@ -150,6 +150,29 @@ cudaError_t launch_encode_f32(RaySoA rays, int64_t M, int L, int ld, float* out,
 cudaError_t launch_sgemm_relu(const float* A, const float* W, const float* b, float* C, int M,
                               int N, int K, cudaStream_t s);
 
+// FP32 layer on the tensor cores (tc_gemm_f32.cu): ReLU(A W^T + b) with both
+// operands given as three bf16 planes that add up to the FP32 values. tmA maps
+// A's planes as one [3 M x K] matrix, tmB W's as [3 N x K], with 128-row boxes;
+// N % 256 == 0. The output is either the next layer's planes [3][M x N] or
+// FP32 rows [M x N]; both and bias 16-byte aligned.
+struct TcF32Params {
+  int M, N, K;
+  const float* bias;
+  __nv_bfloat16* out_planes;  // exactly one of the two outputs is set
+  float* out_f32;
+  uint32_t* status;
+  uint64_t timeout_ns;
+};
+cudaError_t launch_tc_gemm_f32(const CUtensorMap& tmA, const CUtensorMap& tmB,
+                               const TcF32Params& p, int clusters, cudaStream_t s);
+int tc_gemm_f32_max_clusters();
+// The encoded rays as planes [3][M x ld], and the planes [3][N x ldd] of
+// src [N x K] zero-padded to ldd columns (a multiple of 8).
+cudaError_t launch_encode_planes(RaySoA rays, int64_t M, int L, int ld, __nv_bfloat16* out,
+                                 cudaStream_t s);
+cudaError_t launch_pack_planes(const float* src, int N, int K, int ldd, __nv_bfloat16* dst,
+                               cudaStream_t s);
+
 // Heads: z = Wo h + bo, t = softplus(z0), vis = sigmoid(z1), optional shadow.
 struct HeadOut {
   float* t;           // nullable

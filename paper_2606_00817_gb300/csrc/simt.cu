@@ -8,8 +8,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
-#include "kernels.h"
+#include "f32_split.cuh"
 #include "heads.cuh"
+#include "kernels.h"
 
 namespace ddf {
 
@@ -41,6 +42,22 @@ __device__ __forceinline__ void store8(__nv_bfloat16* dst, const float* src) {
 __device__ __forceinline__ void store8(float* dst, const float* src) {
   reinterpret_cast<float4*>(dst)[0] = make_float4(src[0], src[1], src[2], src[3]);
   reinterpret_cast<float4*>(dst)[1] = make_float4(src[4], src[5], src[6], src[7]);
+}
+
+// Three bf16 planes of an FP32 row, `plane` elements apart (element type tag).
+struct F32Planes {
+  __nv_bfloat16 v;
+};
+template <typename T>
+__device__ __forceinline__ void store_row8(T* out, int64_t at, int64_t, const float* src) {
+  store8(out + at, src);
+}
+__device__ __forceinline__ void store_row8(F32Planes* out, int64_t at, int64_t plane,
+                                           const float* src) {
+  uint4 w[3];
+  f32_split8(src, w);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) *reinterpret_cast<uint4*>(out + at + j * plane) = w[j];
 }
 
 constexpr int kEncRays = 64;  // rays per block of the encoder
@@ -83,11 +100,10 @@ __global__ void __launch_bounds__(kEncRays) encode_kernel(RaySoA rays, int64_t M
   // on consecutive chunks. ld is a multiple of 8.
   const int per_row = ld / 8;
   const int total = rows * per_row;
-  T* dst = out + r0 * ld;
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
     const int r = idx / per_row;
     const int c = (idx - r * per_row) * 8;
-    store8(dst + static_cast<int64_t>(r) * ld + c, enc_smem + r * sld + c);
+    store_row8(out, (r0 + r) * ld + c, M * ld, enc_smem + r * sld + c);
   }
 }
 
@@ -309,6 +325,11 @@ cudaError_t launch_encode_bf16(RaySoA rays, int64_t M, int L, int ld, __nv_bfloa
 
 cudaError_t launch_encode_f32(RaySoA rays, int64_t M, int L, int ld, float* out, cudaStream_t s) {
   return launch_encode<float>(rays, M, L, ld, out, s);
+}
+
+cudaError_t launch_encode_planes(RaySoA rays, int64_t M, int L, int ld, __nv_bfloat16* out,
+                                 cudaStream_t s) {
+  return launch_encode<F32Planes>(rays, M, L, ld, reinterpret_cast<F32Planes*>(out), s);
 }
 
 cudaError_t launch_sgemm_relu(const float* A, const float* W, const float* b, float* C, int M,
