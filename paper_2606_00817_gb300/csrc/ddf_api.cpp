@@ -330,6 +330,24 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
   const int W = h->cfg.width;
   const int H = h->cfg.hidden_layers;
   const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
+  if (h->narrow && h->tile_auto) {
+    ddf::NarrowMaps maps{};
+    ddf::NarrowParams p{};
+    p.M = m;
+    p.L = h->cfg.octaves;
+    p.H = H;
+    for (int l = 0; l < H; ++l) {
+      maps.m[l] = h->tmNarrow[l];
+      p.bias[l] = h->bias[l];
+    }
+    p.head_w = h->head_w;
+    p.head_b = h->head_b;
+    p.status = h->status_dev;
+    p.timeout_ns = h->timeout_ns;
+    ProfScope ps(h, kProfGemm, st);
+    DDF_CK(ddf::launch_tc_narrow(maps, p, rays, out, W, h->num_sms, st));
+    return DDF_OK;
+  }
   // layer 1 may build the encoding itself (ddf_set_tile checked the shape)
   const bool fused1 = h->tile_first.fused && h->cfg.kind == DDF_KIND_RAY;
   if (!fused1) {
@@ -772,6 +790,8 @@ ddf_status ddf_create(const ddf_config* cfg, ddf_handle* out) {
   if (layered && cfg->precision == DDF_FP32 && cfg->width % 256 == 0 && major == 10 &&
       minor == 3 && get_encode_fn() != nullptr)
     h->f32_clusters = ddf::tc_gemm_f32_max_clusters();
+  h->narrow = cfg->kind == DDF_KIND_RAY && cfg->precision == DDF_BF16 &&
+              ddf::tc_narrow_supported(cfg->octaves, cfg->width, cfg->hidden_layers);
   cudaError_t e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
   void* p = nullptr;
   if (e != cudaSuccess || dev_alloc(h, &p, sizeof(uint32_t)) != DDF_OK) {
@@ -849,6 +869,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     h->wcal.assign(H, nullptr);
     h->tmB.assign(H, CUtensorMap{});
     h->tmBcal.assign(H, CUtensorMap{});
+    h->tmNarrow.assign(H, CUtensorMap{});
     for (int l = 0; l < H; ++l) {
       const int K = l == 0 ? h->d_in : W;
       if ((s = dev_alloc(h, &p, W * sizeof(float))) != DDF_OK) return s;
@@ -872,6 +893,9 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
         h->wb[l] = static_cast<__nv_bfloat16*>(p);
         if (!make_tmap(&h->tmB[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2,
                        (l == 0 ? h->tile_first : h->tile).pair ? 128u : (l == 0 ? h->tile_first : h->tile).bn))
+          return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+        if (h->narrow && !make_tmap(&h->tmNarrow[l], h->wb[l], false, kp, W,
+                                    static_cast<uint64_t>(kp) * 2, static_cast<uint32_t>(W)))
           return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
       } else {
         if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * W)) != DDF_OK) return s;
@@ -1351,6 +1375,7 @@ ddf_status ddf_set_tile(ddf_handle h, int32_t which, const ddf_tile* tile) {
   (which == 1 ? h->tile_first : h->tile) =
       ddf::TcTile{bn, ew, tile->cta_pair != 0, tile->staged != 0, tile->fused_encode != 0};
   h->bn = h->tile.bn;
+  h->tile_auto = false;
   if (h->loaded && h->cfg.precision != DDF_FP32) {
     DeviceGuard g(h->cfg.device);
     DDF_CK(cudaDeviceSynchronize());  // launches in flight keep their own copies of the maps
@@ -1410,7 +1435,7 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
   ddf_tile keep_h, keep_f;
   ddf_get_tile(h, 0, &keep_h);
   ddf_get_tile(h, 1, &keep_f);
-  const bool keep_prof = h->prof;
+  const bool keep_prof = h->prof, keep_auto = h->tile_auto;
   h->prof = false;
   bool have_ref = false;
   ddf_status result = DDF_OK;
@@ -1508,6 +1533,25 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
     result = ddf_set_tile(h, 0, &kCands[best_h]);
     if (result == DDF_OK) best_f = tune(0, kTileCands, true, p2);
   }
+  // a narrow field's one-kernel query, against the tiles just chosen
+  bool fused_wins = false;
+  if (result == DDF_OK && best_f >= 0 && h->narrow &&
+      (result = ddf_set_tile(h, 1, &kCands[best_f])) == DDF_OK) {
+    double layered = 1e30, fused = 1e30;
+    bool pass = false;
+    h->tile_auto = true;
+    result = check(&pass);
+    for (int round = 0; round < kRounds && result == DDF_OK && pass; ++round) {
+      double a = 0.0, b = 0.0;
+      if ((result = timed(false, &a)) != DDF_OK) break;
+      h->tile_auto = false;
+      if ((result = timed(false, &b)) != DDF_OK) break;
+      h->tile_auto = true;
+      fused = std::min(fused, a);
+      layered = std::min(layered, b);
+    }
+    fused_wins = pass && fused <= layered;
+  }
   for (int c = 0; ms_out != nullptr && c < kTileCands; ++c) {
     ms_out[c] = p1[c];
     ms_out[kTileCands + c] = p2[c];
@@ -1517,10 +1561,13 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
   if (result != DDF_OK || best_h < 0 || best_f < 0) {
     ddf_set_tile(h, 0, &keep_h);
     ddf_set_tile(h, 1, &keep_f);
+    h->tile_auto = keep_auto;
     return result != DDF_OK ? result : fail(DDF_ERR_CUDA, "autotune: no candidate passed");
   }
   ddf_status r = ddf_set_tile(h, 0, &kCands[best_h]);
-  return r != DDF_OK ? r : ddf_set_tile(h, 1, &kCands[best_f]);
+  if (r == DDF_OK) r = ddf_set_tile(h, 1, &kCands[best_f]);
+  h->tile_auto = r == DDF_OK && fused_wins;
+  return r;
 }
 
 }  // extern "C"

@@ -35,6 +35,11 @@ struct ddf_s {
   int bn = 0;    // tensor-core N tile (= tile.bn)
   ddf::TcTile tile{256, 4};        // layers 2..H
   ddf::TcTile tile_first{256, 4};  // layer 1
+  // narrow bf16 ray fields: the whole query in one kernel (tc_narrow.cu), unless
+  // tiles were set by the caller or found faster by the autotuner
+  bool narrow = false;
+  bool tile_auto = true;
+  std::vector<CUtensorMap> tmNarrow;
   int pair_clusters = 0;  // co-resident clusters of the CTA-pair kernel
   int num_sms = 0;
   bool loaded = false;

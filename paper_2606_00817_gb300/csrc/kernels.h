@@ -173,6 +173,26 @@ cudaError_t launch_encode_planes(RaySoA rays, int64_t M, int L, int ld, __nv_bfl
 cudaError_t launch_pack_planes(const float* src, int N, int K, int ldd, __nv_bfloat16* dst,
                                cudaStream_t s);
 
+// A whole bf16 ray query of a narrow field in one kernel (tc_narrow.cu): width
+// 128 or 256, 1 .. kNarrowLayers hidden layers, every weight matrix mapped with
+// boxes of 64 K x `width` rows. The same bits as the default layer tiles.
+constexpr int kNarrowLayers = 16;
+struct NarrowMaps {
+  CUtensorMap m[kNarrowLayers];
+};
+struct NarrowParams {
+  int M, L, H;
+  const float* bias[kNarrowLayers];
+  const float* head_w;  // [2 x width]
+  const float* head_b;  // [2]
+  uint32_t* status;
+  uint64_t timeout_ns;
+};
+struct HeadOut;
+bool tc_narrow_supported(int L, int W, int H);
+cudaError_t launch_tc_narrow(const NarrowMaps& maps, const NarrowParams& p, const RaySoA& rays,
+                             const HeadOut& out, int W, int num_sms, cudaStream_t st);
+
 // Heads: z = Wo h + bo, t = softplus(z0), vis = sigmoid(z1), optional shadow.
 struct HeadOut {
   float* t;           // nullable
