@@ -525,9 +525,10 @@ std::vector<uint64_t> query_key(int kind, const float* const rays[6], int64_t n,
 // Enqueues a query on st: directly, or in graph mode by replaying the CUDA
 // graph captured (on a private stream) the first time this key was seen.
 // Workspaces must already be large enough: nothing is allocated while capturing.
-template <class F>
-ddf_status enqueue(ddf_s* h, const std::vector<uint64_t>& key, cudaStream_t st, F body) {
+template <class K, class F>
+ddf_status enqueue(ddf_s* h, K make_key, cudaStream_t st, F body) {
   if (!h->graph_mode) return body(st);
+  const std::vector<uint64_t> key = make_key();
   for (auto& g : h->graphs) {
     if (g.key == key) {
       DDF_CK(cudaGraphLaunch(g.exec, st));
@@ -1021,7 +1022,7 @@ ddf_status ddf_query_rays(ddf_handle h, const float* const rays[6], int64_t n, f
   ddf::HeadOut o{};
   o.t = out_t;
   o.vis = out_vis;
-  return enqueue(h, query_key(0, rays, n, {out_t, out_vis}, nullptr, 0),
+  return enqueue(h, [&] { return query_key(0, rays, n, {out_t, out_vis}, nullptr, 0); },
                  static_cast<cudaStream_t>(stream),
                  [&](cudaStream_t st) { return run_query(h, rays, n, o, st); });
 }
@@ -1045,7 +1046,7 @@ ddf_status ddf_query_shadow(ddf_handle h, const float* const rays[6], int64_t n,
   o.vis = out_vis;
   o.occluded = out_occluded;
   for (int i = 0; i < 3; ++i) o.light[i] = light[i];
-  return enqueue(h, query_key(1, rays, n, {out_t, out_vis, out_occluded}, light, 0),
+  return enqueue(h, [&] { return query_key(1, rays, n, {out_t, out_vis, out_occluded}, light, 0); },
                  static_cast<cudaStream_t>(stream),
                  [&](cudaStream_t st) { return run_query(h, rays, n, o, st); });
 }
@@ -1071,7 +1072,7 @@ ddf_status ddf_query_ao(ddf_handle h, const float* const rays[6], int64_t n_rays
   ddf::HeadOut o{};
   o.vis = h->ao_vis;
   o.hit = h->ao_hit;
-  return enqueue(h, query_key(2, rays, n_rays, {offsets, out_hard, out_soft}, nullptr, n_points),
+  return enqueue(h, [&] { return query_key(2, rays, n_rays, {offsets, out_hard, out_soft}, nullptr, n_points); },
                  static_cast<cudaStream_t>(stream), [&](cudaStream_t st) {
                    ddf_status r = n_rays > 0 ? run_query(h, rays, n_rays, o, st) : DDF_OK;
                    if (r != DDF_OK) return r;
@@ -1130,7 +1131,7 @@ ddf_status ddf_query_mixed(ddf_handle h, const float* const shadow_rays[6], int6
        r.q[4], r.q[5]},
       n_shadow > 0 ? light : nullptr, n_points);
   key.push_back(static_cast<uint64_t>(n_shadow));
-  return enqueue(h, key, static_cast<cudaStream_t>(stream), [&](cudaStream_t st) {
+  return enqueue(h, [&] { return key; }, static_cast<cudaStream_t>(stream), [&](cudaStream_t st) {
     ddf_status q = n > 0 ? run_query_soa(h, r, n, o, st) : DDF_OK;
     if (q != DDF_OK) return q;
     DDF_CK(ddf::launch_ao_reduce(h->ao_hit, h->ao_vis, offsets, n_points, out_hard, out_soft, st));
