@@ -39,7 +39,7 @@ struct ddf_s {
   // tiles were set by the caller or found faster by the autotuner
   bool narrow = false;
   bool tile_auto = true;
-  std::vector<CUtensorMap> tmNarrow;
+  CUtensorMap* narrow_maps = nullptr;  // device: a launch does not carry 2 KB of maps
   int pair_clusters = 0;  // co-resident clusters of the CTA-pair kernel
   int num_sms = 0;
   bool loaded = false;

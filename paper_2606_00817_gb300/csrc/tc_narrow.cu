@@ -65,7 +65,7 @@ NwShape nw_shape(int L, int W, int H) {
   s.a_bytes = kNwBlock * (s.kb1 > W / 64 ? s.kb1 : W / 64);
   const int chunk = W * 128;
   const int chunks = s.kb1 + (H - 1) * (W / 64);
-  const int vec = (H * W + 2 * W + 4) * 4;
+  const int vec = (H * W + 2 * W + 4 + 2 * 128) * 4;
   for (int g = W == 128 ? 2 : 1; g >= 1; --g) {
     const int room = (kNwSmemMax - kNwCtrl - vec - g * s.a_bytes) / chunk;
     s.groups = g;
@@ -80,8 +80,8 @@ NwShape nw_shape(int L, int W, int H) {
 
 template <int W>
 __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
-    tc_narrow_kernel(const __grid_constant__ NarrowMaps maps, const NarrowParams p,
-                     const NwShape sh, const RaySoA rays, const HeadOut out) {
+    tc_narrow_kernel(const __grid_constant__ NarrowParams p, const NwShape sh,
+                     const __grid_constant__ RaySoA rays, const __grid_constant__ HeadOut out) {
   constexpr int kChunk = W * 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -95,12 +95,33 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kNwSlots + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* sbias = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kNwCtrl);
-  float* shw = sbias + p.H * W;  // two head rows, then the head bias
+  float* shw = sbias + p.H * W;  // two head rows, then the head bias (4 floats)
+  float* sz = shw + 2 * W + 4;   // z1 of each group's rows
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int groups = sh.groups;
   const bool producer = warp == groups * (kNwGroup / 32);
 
-  if (tid == 0) {
+  const int64_t tiles = (p.M + 127) / 128;
+  const int kbh = W / 64;                       // K blocks of a hidden layer
+  const int chunks = sh.kb1 + (p.H - 1) * kbh;  // of one tile
+
+  // The producer thread: barriers, then weight chunks for as long as the ring
+  // has room, before the rest of the CTA is even set up.
+  int64_t loaded = 0;  // chunks issued
+  int load_layer = 0, load_kb = 0;
+  auto load_chunk = [&]() {
+    const int s = static_cast<int>(loaded % sh.slots);
+    mbar_arrive_expect_tx(full_bar(s), kChunk);
+    tma_load_2d(smem_u32(ring + s * kChunk), p.maps + load_layer, load_kb * 64, 0, full_bar(s));
+    ++loaded;
+    if (++load_kb == (load_layer == 0 ? sh.kb1 : kbh)) {
+      load_kb = 0;
+      load_layer = load_layer + 1 == p.H ? 0 : load_layer + 1;
+    }
+  };
+  int64_t total = 0;  // chunks this CTA needs
+  if (producer && lane == 0) {
+    for (int l = 0; l < p.H; ++l) tma_prefetch_desc(p.maps + l);
     for (int s = 0; s < sh.slots; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
@@ -108,15 +129,69 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
     for (int g = 0; g < groups; ++g) mbar_init(done_bar(g), 1);
     *abort_flag = 0;
     fence_mbar_init();
+    // tiles of this CTA pass through its groups in turn; a streamed field has one group
+    const int64_t mine = tiles > blockIdx.x ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    total = sh.resident ? (mine > 0 ? chunks : 0) : mine * chunks;
+    while (loaded < total && loaded < sh.slots) load_chunk();
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(tmem_slot), groups * W);
     tmem_relinquish();
   }
-  for (int l = 0; l < p.H; ++l)
-    for (int i = tid; i < W; i += blockDim.x) sbias[l * W + i] = __ldg(p.bias[l] + i);
-  for (int i = tid; i < 2 * W; i += blockDim.x) shw[i] = __ldg(p.head_w + i);
-  if (tid < 2) shw[2 * W + tid] = __ldg(p.head_b + tid);
+  {  // biases, head rows and head bias, all loads of a round in flight at once
+    const int nb = p.H * W, nv = nb + 2 * W + 2;
+    for (int i0 = tid; i0 < nv; i0 += 4 * blockDim.x) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * blockDim.x;
+        if (i < nv)
+          v[j] = __ldg(i < nb ? p.bias[i / W] + i % W
+                              : i < nb + 2 * W ? p.head_w + (i - nb) : p.head_b + (i - nb - 2 * W));
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * blockDim.x;
+        if (i < nv) sbias[i] = v[j];
+      }
+    }
+  }
+
+  // Encodes the rays of `tile` into group g's operand tile: 2 threads a ray, 3
+  // coordinates each.
+  const int g = warp >> 3;
+  const int gt = tid - g * kNwGroup;  // thread of the group
+  uint8_t* const sA = smem + g * sh.a_bytes;
+  auto encode = [&](int64_t tile) {
+    const int er = gt & 127, part = gt >> 7;
+    const int64_t row = tile * 128 + er;
+    float e[3] = {0.f, 0.f, 0.f};
+    if (row < p.M) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) e[c] = ray_ld(rays, 3 * part + c, row);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int col = 3 * part + c;
+      *reinterpret_cast<__nv_bfloat16*>(sA + nw_off(er, col & ~1) + ((col & 1) << 1)) =
+          __float2bfloat16_rn(e[c]);
+    }
+    for (int k = 0; k < p.L; ++k) {  // three independent chains at a time
+      const float f = __int_as_float((127 + k) << 23);  // 2^k exactly
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float sn, cs;
+        sincospif(e[c] * f, &sn, &cs);
+        *reinterpret_cast<uint32_t*>(sA + nw_off(er, 6 + 2 * ((3 * part + c) * p.L + k))) =
+            epi_pack_bf16x2(sn, cs);
+      }
+    }
+    if (part == 0)
+      for (int col = 6 + 12 * p.L; col < sh.kb1 * 64; col += 2)
+        *reinterpret_cast<uint32_t*>(sA + nw_off(er, col)) = 0u;
+  };
+  const int64_t tile0 = blockIdx.x + static_cast<int64_t>(gridDim.x) * g;
+  if (!producer && tile0 < tiles) encode(tile0);  // beside the first loads
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -126,42 +201,25 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
     atomicOr(p.status, kStatusPipelineTimeout);
   };
 
-  const int64_t tiles = (p.M + 127) / 128;
-  const int kbh = W / 64;                            // K blocks of a hidden layer
-  const int chunks = sh.kb1 + (p.H - 1) * kbh;       // of one tile
-
   if (producer) {
     if (lane == 0) {
-      // tiles of this CTA pass through its groups in turn; a streamed field has one group
-      const int64_t mine = tiles > blockIdx.x ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-      const int64_t total = sh.resident ? (mine > 0 ? chunks : 0) : mine * chunks;
       bool ok = true;
-      int64_t it = 0;
-      int layer = 0, kb = 0;
-      for (; it < total; ++it) {
-        const int s = static_cast<int>(it % sh.slots);
-        const uint32_t ph = static_cast<uint32_t>((it / sh.slots) & 1);
+      while (loaded < total) {
+        const int s = static_cast<int>(loaded % sh.slots);
+        const uint32_t ph = static_cast<uint32_t>((loaded / sh.slots) & 1);
         if (!mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, p.timeout_ns)) {
           ok = false;
           break;
         }
-        mbar_arrive_expect_tx(full_bar(s), kChunk);
-        tma_load_2d(smem_u32(ring + s * kChunk), &maps.m[layer], kb * 64, 0, full_bar(s));
-        if (++kb == (layer == 0 ? sh.kb1 : kbh)) {
-          kb = 0;
-          layer = layer + 1 == p.H ? 0 : layer + 1;
-        }
+        load_chunk();
       }
       if (!ok) raise_abort();
       // no exit with a copy in flight
-      for (int64_t j = it > sh.slots ? it - sh.slots : 0; j < it; ++j)
+      for (int64_t j = loaded > sh.slots ? loaded - sh.slots : 0; j < loaded; ++j)
         mbar_wait_bounded(full_bar(static_cast<int>(j % sh.slots)),
                           static_cast<uint32_t>((j / sh.slots) & 1), nullptr, kNwDrainNs);
     }
   } else {
-    const int g = warp >> 3;
-    const int gt = tid - g * kNwGroup;               // thread of the group
-    uint8_t* sA = smem + g * sh.a_bytes;
     const uint32_t a0 = smem_u32(sA);
     const int q = warp & 3, half = (gt >> 7);        // TMEM lane quarter, column half
     const int r = q * 32 + lane;                     // this thread's row of the accumulator
@@ -186,35 +244,9 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
     int64_t it = 0;       // streamed: chunks consumed
     uint32_t dphase = 0;  // layers finished, mod 2
     bool ok = true;
-    for (int64_t tile = blockIdx.x + static_cast<int64_t>(gridDim.x) * g; tile < tiles && ok;
+    for (int64_t tile = tile0; tile < tiles && ok;
          tile += static_cast<int64_t>(gridDim.x) * groups) {
-      {  // encode: 2 threads a ray, 3 coordinates each
-        const int er = gt & 127, part = gt >> 7;
-        const int64_t row = tile * 128 + er;
-        float e[3] = {0.f, 0.f, 0.f};
-        if (row < p.M) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) e[c] = ray_ld(rays, 3 * part + c, row);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int col = 3 * part + c;
-          *reinterpret_cast<__nv_bfloat16*>(sA + nw_off(er, col & ~1) + ((col & 1) << 1)) =
-              __float2bfloat16_rn(e[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          int col = 6 + 2 * (3 * part + c) * p.L;
-          for (int k = 0; k < p.L; ++k, col += 2) {
-            float sn, cs;
-            sincospif(e[c] * __int_as_float((127 + k) << 23), &sn, &cs);  // 2^k exactly
-            *reinterpret_cast<uint32_t*>(sA + nw_off(er, col)) = epi_pack_bf16x2(sn, cs);
-          }
-        }
-        if (part == 0)
-          for (int col = 6 + 12 * p.L; col < sh.kb1 * 64; col += 2)
-            *reinterpret_cast<uint32_t*>(sA + nw_off(er, col)) = 0u;
-      }
+      if (tile != tile0) encode(tile);
       for (int l = 0; l < p.H; ++l) {
         fence_proxy_async_smem();  // this thread's part of the tile, for the MMAs
         tc_fence_before();
@@ -239,11 +271,10 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
             if (!sh.resident) tc_commit(empty_bar(s));
           }
           tc_commit(done_bar(g));  // arrives once every MMA above has finished
+          ok = mbar_wait_bounded(done_bar(g), dphase, nullptr, p.timeout_ns) && ok;
         }
-        // the group goes on, or gives up, together
-        ok = mbar_wait_bounded(done_bar(g), dphase, nullptr, p.timeout_ns) && ok;
         dphase ^= 1u;
-        ok = group_and(ok);
+        ok = group_and(ok);  // the group goes on, or gives up, together
         if (!ok) break;
         tc_fence_after();
         if (l + 1 < p.H) {  // ReLU(acc + b) in bf16 over the tile: the next operand
@@ -266,15 +297,33 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
               *reinterpret_cast<uint4*>(sA + nw_off(r, col + 8 * k)) = w;
             }
           }
-        } else if (half == 0) {  // the FP32 head, column by column
-          TcGemmParams hp{};
-          hp.mode = 1;
-          const EpiVectors ev{sbias + l * W, nullptr, shw, shw + W, 1.f};
-          float h0 = 0.f, h1 = 0.f;
-          epi_row<false, true>(hp, ev, trow, 0, true, 0, 0, W / 32, h0, h1);
+        } else {
+          // the FP32 head, column by column: z0 by the threads of half 0, z1 by
+          // those of half 1, which pass it on through shared memory
+          const float* hw = shw + half * W;
+          const float* bias = sbias + l * W;
+          float z = 0.f;
+#pragma unroll 1
+          for (int c = 0; c < W / 32; ++c) {
+            uint32_t v[32];
+            tmem_ld32(trow + 32 * c, v);
+            tmem_wait_ld_regs(v);
+            const float4* b4 = reinterpret_cast<const float4*>(bias + 32 * c);
+            const float4* w4 = reinterpret_cast<const float4*>(hw + 32 * c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const float4 b = b4[k], w = w4[k];
+              z = fmaf(fmaxf(__uint_as_float(v[4 * k + 0]) + b.x, 0.f), w.x, z);
+              z = fmaf(fmaxf(__uint_as_float(v[4 * k + 1]) + b.y, 0.f), w.y, z);
+              z = fmaf(fmaxf(__uint_as_float(v[4 * k + 2]) + b.z, 0.f), w.z, z);
+              z = fmaf(fmaxf(__uint_as_float(v[4 * k + 3]) + b.w, 0.f), w.w, z);
+            }
+          }
+          z = (0.f + z) + shw[2 * W + half];
+          if (half == 1) sz[g * 128 + r] = z;
+          group_sync();
           const int64_t row = tile * 128 + r;
-          if (row < p.M)
-            write_heads(out, row, (0.f + h0) + shw[2 * W], (0.f + h1) + shw[2 * W + 1]);
+          if (half == 0 && row < p.M) write_heads(out, row, z, sz[g * 128 + r]);
         }
       }
       // the accumulator is read before the next tile's MMAs
@@ -295,14 +344,14 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
 }
 
 template <int W>
-cudaError_t launch_w(const NarrowMaps& maps, const NarrowParams& p, const NwShape& s,
+cudaError_t launch_w(const NarrowParams& p, const NwShape& s,
                      const RaySoA& rays, const HeadOut& out, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(tc_narrow_kernel<W>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (p.M + 127) / 128;
   const int grid = static_cast<int>(tiles < num_sms ? tiles : num_sms);
-  tc_narrow_kernel<W><<<grid, s.groups * kNwGroup + 32, s.smem, st>>>(maps, p, s, rays, out);
+  tc_narrow_kernel<W><<<grid, s.groups * kNwGroup + 32, s.smem, st>>>(p, s, rays, out);
   return cudaGetLastError();
 }
 
@@ -312,13 +361,13 @@ bool tc_narrow_supported(int L, int W, int H) {
   return (W == 128 || W == 256) && H >= 1 && H <= kNarrowLayers && nw_shape(L, W, H).slots > 0;
 }
 
-cudaError_t launch_tc_narrow(const NarrowMaps& maps, const NarrowParams& p, const RaySoA& rays,
-                             const HeadOut& out, int W, int num_sms, cudaStream_t st) {
+cudaError_t launch_tc_narrow(const NarrowParams& p, const RaySoA& rays, const HeadOut& out, int W,
+                             int num_sms, cudaStream_t st) {
   if (p.M <= 0) return cudaSuccess;
   if (!tc_narrow_supported(p.L, W, p.H)) return cudaErrorInvalidValue;
   const NwShape s = nw_shape(p.L, W, p.H);
-  return W == 128 ? launch_w<128>(maps, p, s, rays, out, num_sms, st)
-                  : launch_w<256>(maps, p, s, rays, out, num_sms, st);
+  return W == 128 ? launch_w<128>(p, s, rays, out, num_sms, st)
+                  : launch_w<256>(p, s, rays, out, num_sms, st);
 }
 
 }  // namespace ddf
