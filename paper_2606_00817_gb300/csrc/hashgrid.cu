@@ -292,251 +292,360 @@ __global__ void __launch_bounds__(kHgRows, 4)  // 4 CTAs per SM: 128 registers
 
 // ------------------------------------------------------------ FP32 path
 
-constexpr int kHgF32Rays = 64;  // rays per block
-constexpr int kHgLd = kHgW + 1; // per-thread row stride in shared memory
+// The FP32 MLP reads its weights from shared memory, transposed ([k][64],
+// rows kHgLdw apart: 16-byte aligned, and the transposing stores spread over
+// the banks), so that one 16-byte load brings the weights of one input to four
+// outputs. Every output is still summed over its inputs in order, in FP32 FMAs.
+constexpr int kHgLdw = kHgW + 4;
 
-// Queries, thread = ray: code and activations in a per-thread shared-memory
-// row, weights broadcast from shared memory, FFMA only.
-__global__ void __launch_bounds__(kHgF32Rays)
-    hashgrid_f32_kernel(const HashGridParams g, const float2* __restrict__ table,
-                        const float* __restrict__ mlp, int H, RaySoA rays, int64_t M,
-                        HeadOut out) {
-  extern __shared__ float fsm[];
-  const int n_mlp = kHgW * kHgCode + kHgW + (H - 1) * (kHgW * kHgW + kHgW) + 2 * kHgW + 2;
-  float* sw = fsm;
-  float* bufA = fsm + ((n_mlp + 3) & ~3);
-  float* bufB = bufA + kHgF32Rays * kHgLd;
-  for (int i = threadIdx.x; i < n_mlp; i += blockDim.x) sw[i] = mlp[i];
-  __syncthreads();
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kHgF32Rays + threadIdx.x;
-  if (row >= M) return;
-  float* a = bufA + threadIdx.x * kHgLd;
-  float* nb = bufB + threadIdx.x * kHgLd;
-  const float x = box01(rays.p[0][row]), y = box01(rays.p[1][row]), z = box01(rays.p[2][row]);
-  auto fetch = [&](uint32_t e0, uint32_t e1, float2& v0, float2& v1) {
-    v0 = __ldg(table + e0);
-    v1 = __ldg(table + e1);
-  };
-  for (int l = 0; l < 16; ++l) hg_level(g, l, x, y, z, fetch, a[2 * l], a[2 * l + 1]);
-  float dcode[27];
-  hg_dir_code(rays.p[3][row], rays.p[4][row], rays.p[5][row], dcode);
-#pragma unroll
-  for (int k = 0; k < 27; ++k) a[32 + k] = dcode[k];
-  const float* w = sw;
-  int K = kHgCode;
+__host__ __device__ constexpr int hg_mlp_floats(int H) {  // the blob's MLP part
+  return kHgW * kHgCode + kHgW + (H - 1) * (kHgW * kHgW + kHgW) + 2 * kHgW + 2;
+}
+// Shared-memory floats of the transposed MLP: per layer K rows and the bias,
+// then the head rows and bias (2 floats, padded to 4).
+__host__ __device__ constexpr int hg_wt_floats(int H) {
+  return (kHgCode + (H - 1) * kHgW) * kHgLdw + H * kHgW + 2 * kHgW + 4;
+}
+
+// Fills that layout from the blob's MLP part; all threads.
+__device__ __forceinline__ void hg_stage_wt(const float* __restrict__ mlp, int H, float* sw) {
+  int src = 0, dst = 0;
   for (int l = 0; l < H; ++l) {
-    const float* b = w + kHgW * K;
-    for (int n = 0; n < kHgW; n += 4) {  // 4 outputs at a time: 4 independent FMA chains
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      const float* w0 = w + n * K;
-      for (int k = 0; k < K; ++k) {
-        const float av = a[k];
-        s0 = fmaf(av, w0[k], s0);
-        s1 = fmaf(av, w0[K + k], s1);
-        s2 = fmaf(av, w0[2 * K + k], s2);
-        s3 = fmaf(av, w0[3 * K + k], s3);
-      }
-      nb[n] = fmaxf(s0 + b[n], 0.f);
-      nb[n + 1] = fmaxf(s1 + b[n + 1], 0.f);
-      nb[n + 2] = fmaxf(s2 + b[n + 2], 0.f);
-      nb[n + 3] = fmaxf(s3 + b[n + 3], 0.f);
+    const int K = l == 0 ? kHgCode : kHgW;
+    if (l == 0) {
+#pragma unroll 8
+      for (int i = threadIdx.x; i < kHgW * kHgCode; i += blockDim.x)
+        sw[(i % kHgCode) * kHgLdw + i / kHgCode] = __ldg(mlp + i);
+    } else {
+#pragma unroll 8
+      for (int i = threadIdx.x; i < kHgW * kHgW; i += blockDim.x)
+        sw[dst + (i % kHgW) * kHgLdw + i / kHgW] = __ldg(mlp + src + i);
     }
-    float* t = a;
-    a = nb;
-    nb = t;
-    w = b + kHgW;
-    K = kHgW;
+    src += kHgW * K;
+    dst += K * kHgLdw;
+    for (int i = threadIdx.x; i < kHgW; i += blockDim.x) sw[dst + i] = __ldg(mlp + src + i);
+    src += kHgW;
+    dst += kHgW;
   }
-  float z0 = 0.f, z1 = 0.f;
-  for (int k = 0; k < kHgW; ++k) {
-    z0 = fmaf(a[k], w[k], z0);
-    z1 = fmaf(a[k], w[kHgW + k], z1);
+  for (int i = threadIdx.x; i < 2 * kHgW + 2; i += blockDim.x) sw[dst + i] = __ldg(mlp + src + i);
+}
+
+// The two x-neighbour entries e0, e1 of an FP32 table: one 16-byte load when
+// both sit in the same aligned pair.
+__device__ __forceinline__ void hg_fetch_f32(const float2* __restrict__ table, uint32_t e0,
+                                             uint32_t e1, float2& v0, float2& v1) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(table) + (e0 >> 1));
+  v0 = (e0 & 1u) ? make_float2(a.z, a.w) : make_float2(a.x, a.y);
+  if ((e1 >> 1) == (e0 >> 1)) v1 = (e1 & 1u) ? make_float2(a.z, a.w) : make_float2(a.x, a.y);
+  else v1 = __ldg(table + e1);
+}
+
+constexpr int kHgF32Rays = 128;     // rays of a query block
+constexpr int kHgF32Threads = 256;
+constexpr int kHgF32Ctas = 3;       // blocks per SM (shared memory)
+constexpr int kHgF32Ld = kHgF32Rays + 4;
+
+// Queries, persistent blocks of 128 rays. Two threads gather a ray's code (8
+// levels and half of the direction each) into [feature][ray]; then the block
+// computes each layer as a [128 x 64] product, 4 rays x 8 outputs a thread:
+// three 16-byte shared loads for 16 packed FMAs an input. Thread = ray with its
+// 64 sums in registers needed 16 loads for 32 FMAs and ran on the shared-memory
+// port (164 us for 100,003 rays; 315 us before that, with scalar loads); this
+// takes 132 us, about half of it gathers.
+__global__ void __launch_bounds__(kHgF32Threads, kHgF32Ctas)
+    hashgrid_f32_kernel(const __grid_constant__ HashGridParams g, const float2* __restrict__ table,
+                        const float* __restrict__ mlp, int H, const __grid_constant__ RaySoA rays,
+                        int64_t M, const __grid_constant__ HeadOut out) {
+  extern __shared__ __align__(16) float fsm[];
+  float* sw = fsm;
+  float* act = fsm + hg_wt_floats(H);  // [64][kHgF32Ld]
+  const int tid = threadIdx.x;
+  hg_stage_wt(mlp, H, sw);
+  const int r = tid & (kHgF32Rays - 1), part = tid / kHgF32Rays;
+  const int tr = tid & 31, tn = tid >> 5;  // rays 4 tr .., outputs 8 tn ..
+  const int64_t tiles = (M + kHgF32Rays - 1) / kHgF32Rays;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t row = tile * kHgF32Rays + r;
+    const bool valid = row < M;
+    const float x = box01(valid ? __ldg(rays.p[0] + row) : 0.f),
+                y = box01(valid ? __ldg(rays.p[1] + row) : 0.f),
+                z = box01(valid ? __ldg(rays.p[2] + row) : 0.f);
+    auto fetch = [&](uint32_t e0, uint32_t e1, float2& v0, float2& v1) {
+      hg_fetch_f32(table, e0, e1, v0, v1);
+    };
+#pragma unroll 2
+    for (int j = 0; j < kHgLevels / 2; ++j) {
+      const int l = 2 * j + part;
+      float f0, f1;
+      hg_level(g, l, x, y, z, fetch, f0, f1);
+      act[(2 * l) * kHgF32Ld + r] = f0;
+      act[(2 * l + 1) * kHgF32Ld + r] = f1;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // part 0: the coordinates and bands 0, 1; part 1: bands 2, 3
+      const float d = valid ? __ldg(rays.p[3 + c] + row) : 0.f;
+      if (part == 0) act[(32 + c) * kHgF32Ld + r] = d;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float sn, co;
+        sincospif(d * __int_as_float((127 + 2 * part + k) << 23), &sn, &co);
+        act[(35 + 8 * c + 2 * (2 * part + k)) * kHgF32Ld + r] = sn;
+        act[(36 + 8 * c + 2 * (2 * part + k)) * kHgF32Ld + r] = co;
+      }
+    }
+    __syncthreads();
+    const float* w = sw;
+    for (int l = 0; l < H; ++l) {
+      const int K = l == 0 ? kHgCode : kHgW;
+      float2 acc[4][4];  // [ray][output pair]
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+      for (int k = 0; k < K; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(act + k * kHgF32Ld + 4 * tr);
+        const float4 u = *reinterpret_cast<const float4*>(w + k * kHgLdw + 8 * tn);
+        const float4 v = *reinterpret_cast<const float4*>(w + k * kHgLdw + 8 * tn + 4);
+        const float av[4] = {a.x, a.y, a.z, a.w};
+        const float2 wv[4] = {{u.x, u.y}, {u.z, u.w}, {v.x, v.y}, {v.z, v.w}};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            acc[i][j] = __ffma2_rn(make_float2(av[i], av[i]), wv[j], acc[i][j]);
+      }
+      const float* b = w + K * kHgLdw + 8 * tn;
+      __syncthreads();  // every thread has read the inputs
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float* d0 = act + (8 * tn + 2 * j) * kHgF32Ld + 4 * tr;
+        const float b0 = b[2 * j], b1 = b[2 * j + 1];
+        *reinterpret_cast<float4*>(d0) =
+            make_float4(fmaxf(acc[0][j].x + b0, 0.f), fmaxf(acc[1][j].x + b0, 0.f),
+                        fmaxf(acc[2][j].x + b0, 0.f), fmaxf(acc[3][j].x + b0, 0.f));
+        *reinterpret_cast<float4*>(d0 + kHgF32Ld) =
+            make_float4(fmaxf(acc[0][j].y + b1, 0.f), fmaxf(acc[1][j].y + b1, 0.f),
+                        fmaxf(acc[2][j].y + b1, 0.f), fmaxf(acc[3][j].y + b1, 0.f));
+      }
+      w += K * kHgLdw + kHgW;
+      __syncthreads();
+    }
+    if (part == 0 && valid) {
+      float z0 = 0.f, z1 = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < kHgW; ++k) {
+        const float h = act[k * kHgF32Ld + r];
+        z0 = fmaf(h, w[k], z0);
+        z1 = fmaf(h, w[kHgW + k], z1);
+      }
+      write_heads(out, row, z0 + w[2 * kHgW], z1 + w[2 * kHgW + 1]);
+    }
+    __syncthreads();  // the activations are read before the next rays' codes
   }
-  z0 += w[2 * kHgW];
-  z1 += w[2 * kHgW + 1];
-  write_heads(out, row, z0, z1);
 }
 
 // ---------------------------------------------------------------- training
-// Training forward and backward with kHgTrainT = 4 threads per ray (64 rays,
-// 256 threads per block): at the batch sizes of a distillation step (16,384
-// rays) one thread per ray leaves 3-4 warps per SM, every table gather and
-// atomic waiting out its full latency. Thread t of a ray takes levels t,
-// t + 4, t + 8, t + 12 and outputs (or input gradients) t + 4 q; each output
-// is still summed over its inputs in order, so the values are those of one
-// thread per ray (8 threads per ray were measured too, and were no faster). The ray's rows live in shared memory as in the query kernel;
-// __syncwarp orders the threads of a ray (same warp). Threads of rays past
-// the end stay to the end (they take part in __syncwarp) and skip every
-// load and store of their row.
-constexpr int kHgTrainT = 4;
-static_assert(kHgLevels % kHgTrainT == 0 && kHgW % kHgTrainT == 0 && 32 % kHgTrainT == 0,
-              "a ray's threads share a warp and split the levels and outputs evenly");
-constexpr int kHgTrainThreads = kHgF32Rays * kHgTrainT;
+// Training forward and backward: 256 threads for 32 rays, so that the 16,384
+// rays of a distillation step give 512 blocks, 4 to an SM. Gathers and scatters:
+// 8 threads a ray, two levels each. Layers: the block computes a [32 x 64]
+// product from the activations ([feature][ray], rows kHgLda apart) and the
+// weights in shared memory, each thread 2 rays x 4 outputs (a 16-byte and an
+// 8-byte load for 8 FMAs); every output is summed over its inputs in order, so
+// the values are those of one thread per ray. With 4 threads a ray, each
+// loading its 16 weights per input one by one, the forward took 71 us and the
+// backward 61; now 53 and 32, of which the forward's gathers are 31 (asking for
+// the whole table in L2 first gained nothing: 10 us for the 52 MB).
+constexpr int kHgTrainRays = 32;
+constexpr int kHgTrainThreads = 256;
+constexpr int kHgLda = kHgTrainRays + 2;  // 8-byte aligned rows, rays of 16 features on 32 banks
+constexpr int kHgTrainT = kHgTrainThreads / kHgTrainRays;  // threads a ray in gathers: 8
 
-// Forward weight rows in shared memory: odd strides (59, 65), so that the
-// 4 threads of a ray, reading rows t + 4 q of one column, hit 4 banks.
-__host__ __device__ constexpr int hg_train_ldw(int l) { return l == 0 ? kHgCode : kHgW + 1; }
-__host__ __device__ constexpr int hg_train_wfloats(int H) {
-  return kHgW * hg_train_ldw(0) + kHgW + (H - 1) * (kHgW * hg_train_ldw(1) + kHgW) + 2 * kHgW + 2;
+// out = in^T W for the block's rays: thread (tr, tn) sums outputs 4 tn ..
+// 4 tn + 3 of rays 2 tr, 2 tr + 1 over k = 0 .. K - 1; in is [k][kHgLda], w is
+// [k][ldw].
+__device__ __forceinline__ void hg_tile(const float* in, const float* w, int ldw, int K, int tr,
+                                        int tn, float (&acc)[2][4]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const float2 a = *reinterpret_cast<const float2*>(in + k * kHgLda + 2 * tr);
+    const float4 b = *reinterpret_cast<const float4*>(w + k * ldw + 4 * tn);
+    acc[0][0] = fmaf(a.x, b.x, acc[0][0]);
+    acc[0][1] = fmaf(a.x, b.y, acc[0][1]);
+    acc[0][2] = fmaf(a.x, b.z, acc[0][2]);
+    acc[0][3] = fmaf(a.x, b.w, acc[0][3]);
+    acc[1][0] = fmaf(a.y, b.x, acc[1][0]);
+    acc[1][1] = fmaf(a.y, b.y, acc[1][1]);
+    acc[1][2] = fmaf(a.y, b.z, acc[1][2]);
+    acc[1][3] = fmaf(a.y, b.w, acc[1][3]);
+  }
 }
 
-__global__ void __launch_bounds__(kHgTrainThreads)
-    hg_train_fwd_kernel(const HashGridParams g, const float2* __restrict__ table,
-                        const float* __restrict__ mlp, int H, RaySoA rays, int64_t M,
-                        float* __restrict__ code_out, float* __restrict__ acts,
+__global__ void __launch_bounds__(kHgTrainThreads, 4)
+    hg_train_fwd_kernel(const __grid_constant__ HashGridParams g, const float2* __restrict__ table,
+                        const float* __restrict__ mlp, int H, const __grid_constant__ RaySoA rays,
+                        int64_t M, float* __restrict__ code_out, float* __restrict__ acts,
                         float2* __restrict__ z_out) {
-  extern __shared__ float fsm[];
+  extern __shared__ __align__(16) float fsm[];
   float* sw = fsm;
-  float* bufA = fsm + ((hg_train_wfloats(H) + 3) & ~3);
-  float* bufB = bufA + kHgF32Rays * kHgLd;
-  {  // weights: blob layout (W_l [64 x K_l], b_l, ..., W_o [2 x 64], b_o) -> padded rows
-    int src = 0, dst = 0;
-    for (int l = 0; l < H; ++l) {
-      const int K = l == 0 ? kHgCode : kHgW, ldw = hg_train_ldw(l);
-      for (int i = threadIdx.x; i < kHgW * K; i += blockDim.x)
-        sw[dst + (i / K) * ldw + i % K] = mlp[src + i];
-      src += kHgW * K;
-      dst += kHgW * ldw;
-      for (int i = threadIdx.x; i < kHgW; i += blockDim.x) sw[dst + i] = mlp[src + i];
-      src += kHgW;
-      dst += kHgW;
+  float* bufA = fsm + hg_wt_floats(H);
+  float* bufB = bufA + kHgW * kHgLda;
+  const int tid = threadIdx.x;
+  const int64_t row0 = static_cast<int64_t>(blockIdx.x) * kHgTrainRays;
+  {  // code: thread (r, t) of ray r takes levels t and t + 8
+    const int r = tid & 31, t = tid >> 5;
+    const int64_t row = row0 + r;
+    const bool valid = row < M;
+    float f[4] = {0.f, 0.f, 0.f, 0.f};
+    if (valid) {
+      const float x = box01(__ldg(rays.p[0] + row)), y = box01(__ldg(rays.p[1] + row)),
+                  z = box01(__ldg(rays.p[2] + row));
+      auto fetch = [&](uint32_t e0, uint32_t e1, float2& v0, float2& v1) {
+        hg_fetch_f32(table, e0, e1, v0, v1);
+      };
+      hg_level(g, t, x, y, z, fetch, f[0], f[1]);
+      hg_level(g, t + kHgTrainT, x, y, z, fetch, f[2], f[3]);
     }
-    for (int i = threadIdx.x; i < 2 * kHgW + 2; i += blockDim.x) sw[dst + i] = mlp[src + i];
-  }
-  __syncthreads();
-  const int r = threadIdx.x / kHgTrainT, t = threadIdx.x % kHgTrainT;
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kHgF32Rays + r;
-  const bool valid = row < M;
-  float* a = bufA + r * kHgLd;
-  float* nb = bufB + r * kHgLd;
-  if (valid) {
-    const float x = box01(rays.p[0][row]), y = box01(rays.p[1][row]), z = box01(rays.p[2][row]);
-    auto fetch = [&](uint32_t e0, uint32_t e1, float2& v0, float2& v1) {
-      v0 = __ldg(table + e0);
-      v1 = __ldg(table + e1);
-    };
+    hg_stage_wt(mlp, H, sw);
+    bufA[(2 * t) * kHgLda + r] = f[0];
+    bufA[(2 * t + 1) * kHgLda + r] = f[1];
+    bufA[(2 * (t + kHgTrainT)) * kHgLda + r] = f[2];
+    bufA[(2 * (t + kHgTrainT) + 1) * kHgLda + r] = f[3];
+    // direction: warp t < 3 its coordinate, warps 3..7 nothing but the padding
+    if (t < 3) {
+      const float d = valid ? __ldg(rays.p[3 + t] + row) : 0.f;
+      bufA[(32 + t) * kHgLda + r] = d;
 #pragma unroll
-    for (int j = 0; j < kHgLevels / kHgTrainT; ++j) {
-      const int l = t + kHgTrainT * j;
-      hg_level(g, l, x, y, z, fetch, a[2 * l], a[2 * l + 1]);
+      for (int k = 0; k < 4; ++k) {
+        float sn, co;
+        sincospif(d * __int_as_float((127 + k) << 23), &sn, &co);
+        bufA[(35 + 8 * t + 2 * k) * kHgLda + r] = sn;
+        bufA[(36 + 8 * t + 2 * k) * kHgLda + r] = co;
+      }
+    } else if (t < 8) {
+      bufA[(kHgCode + t - 3) * kHgLda + r] = 0.f;  // features 59 .. 63
     }
-    if (t == 0) {
-      float dcode[27];
-      hg_dir_code(rays.p[3][row], rays.p[4][row], rays.p[5][row], dcode);
-#pragma unroll
-      for (int k = 0; k < 27; ++k) a[32 + k] = dcode[k];
-    }
+    static_assert(kHgCode == 59 && kHgTrainT == 8 && kHgLevels == 16, "the code's layout");
+    __syncthreads();
+    for (int k = t; k < kHgW; k += kHgTrainT)
+      if (valid) code_out[k * M + row] = bufA[k * kHgLda + r];
   }
-  __syncwarp();
-  if (valid)
-    for (int k = t; k < kHgW; k += kHgTrainT) code_out[k * M + row] = k < kHgCode ? a[k] : 0.f;
+  const int tr = tid & 15, tn = tid >> 4;
   const float* w = sw;
-  int K = kHgCode;
+  float* a = bufA;
+  float* nb = bufB;
   for (int l = 0; l < H; ++l) {
-    const int ldw = hg_train_ldw(l);
-    const float* b = w + kHgW * ldw;
-    float sacc[kHgW / kHgTrainT];
+    const int K = l == 0 ? kHgCode : kHgW;
+    float acc[2][4];
+    hg_tile(a, w, kHgLdw, K, tr, tn, acc);
+    const float4 b = *reinterpret_cast<const float4*>(w + K * kHgLdw + 4 * tn);
+    const float bb[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int q = 0; q < kHgW / kHgTrainT; ++q) sacc[q] = 0.f;
-    for (int k = 0; k < K; ++k) {
-      const float av = a[k];
-#pragma unroll
-      for (int q = 0; q < kHgW / kHgTrainT; ++q)
-        sacc[q] = fmaf(av, w[(t + kHgTrainT * q) * ldw + k], sacc[q]);
-    }
-    float* dst = acts + static_cast<int64_t>(l) * kHgW * M + row;
-#pragma unroll
-    for (int q = 0; q < kHgW / kHgTrainT; ++q) {
-      const int n = t + kHgTrainT * q;
-      const float hv = fmaxf(sacc[q] + b[n], 0.f);
-      nb[n] = hv;
-      if (valid) dst[n * M] = hv;
-    }
-    __syncwarp();
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<float2*>(nb + (4 * tn + j) * kHgLda + 2 * tr) =
+          make_float2(fmaxf(acc[0][j] + bb[j], 0.f), fmaxf(acc[1][j] + bb[j], 0.f));
+    w += K * kHgLdw + kHgW;
+    __syncthreads();
+    float* dst = acts + static_cast<int64_t>(l) * kHgW * M + row0;
+    const int r = tid & 31;
+    if (row0 + r < M)
+      for (int k = tid >> 5; k < kHgW; k += kHgTrainT) dst[k * M + r] = nb[k * kHgLda + r];
     float* tmp = a;
     a = nb;
     nb = tmp;
-    w = b + kHgW;
-    K = kHgW;
   }
-  if (valid && t == 0) {
-    float z0 = 0.f, z1 = 0.f;
-    for (int k = 0; k < kHgW; ++k) {
-      z0 = fmaf(a[k], w[k], z0);
-      z1 = fmaf(a[k], w[kHgW + k], z1);
-    }
-    z0 += w[2 * kHgW];
-    z1 += w[2 * kHgW + 1];
-    z_out[row] = make_float2(z0, z1);
+  if (tid < 2 * kHgTrainRays) {  // warp 0: z0, warp 1: z1
+    const int r = tid & 31, o = tid >> 5;
+    float z = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < kHgW; ++k) z = fmaf(a[k * kHgLda + r], w[o * kHgW + k], z);
+    z += w[2 * kHgW + o];
+    if (row0 + r < M) reinterpret_cast<float*>(z_out)[2 * (row0 + r) + o] = z;
   }
 }
 
-// Backward of the training forward above, kHgTrainT threads per ray: dL/dpre of
-// every layer (feature-major, [H x 64 x B]) and the hash features' gradient
-// scattered into the level tables' gradient (blob layout, 8-byte aligned):
-// each corner entry receives its trilinear weight times the feature
-// gradient (atomic adds; entries shared by several rays or corners sum up).
-__global__ void __launch_bounds__(kHgTrainThreads)
-    hg_train_bwd_kernel(const HashGridParams g, const float* __restrict__ mlp, int H, RaySoA rays,
-                        int64_t M, const float* __restrict__ acts, const float2* __restrict__ dz,
+// Backward of the training forward above: dL/dpre of every layer
+// (feature-major, [H x 64 x B]) and the hash features' gradient scattered into
+// the level tables' gradient (blob layout, 8-byte aligned): each corner entry
+// receives its trilinear weight times the feature gradient (atomic adds;
+// entries shared by several rays or corners sum up).
+constexpr int kHgLdf = 2 * kHgLevels + 4;  // weight rows of layer 1: the hash features only
+__host__ __device__ constexpr int hg_bwd_floats(int H) {
+  return kHgW * kHgLdf + (H - 1) * kHgW * kHgLdw + 2 * kHgW;
+}
+
+__global__ void __launch_bounds__(kHgTrainThreads, 4)
+    hg_train_bwd_kernel(const __grid_constant__ HashGridParams g, const float* __restrict__ mlp,
+                        int H, const __grid_constant__ RaySoA rays, int64_t M,
+                        const float* __restrict__ acts, const float2* __restrict__ dz,
                         float* __restrict__ dpre, float* __restrict__ grad_table) {
-  extern __shared__ float fsm[];
-  const int n_mlp = kHgW * kHgCode + kHgW + (H - 1) * (kHgW * kHgW + kHgW) + 2 * kHgW + 2;
-  float* sw = fsm;
-  float* bufA = fsm + ((n_mlp + 3) & ~3);
-  float* bufB = bufA + kHgF32Rays * kHgLd;
-  for (int i = threadIdx.x; i < n_mlp; i += blockDim.x) sw[i] = mlp[i];
-  __syncthreads();
-  const int r = threadIdx.x / kHgTrainT, t = threadIdx.x % kHgTrainT;
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * kHgF32Rays + r;
-  const bool valid = row < M;
-  float* dh = bufA + r * kHgLd;
-  float* dn = bufB + r * kHgLd;
-  // weight offsets: layer l's W [64 x K_l] and b, then the head W_o [2 x 64], b_o
-  int woff[4];
-  int off = 0;
-  for (int l = 0; l < H; ++l) {
-    woff[l] = off;
-    off += kHgW * (l == 0 ? kHgCode : kHgW) + kHgW;
+  extern __shared__ __align__(16) float fsm[];
+  float* sw = fsm;  // W_1's hash columns [64][kHgLdf], W_l [64][kHgLdw] ..., head rows
+  float* bufA = fsm + hg_bwd_floats(H);
+  float* bufB = bufA + kHgW * kHgLda;
+  const int tid = threadIdx.x;
+  const int64_t row0 = static_cast<int64_t>(blockIdx.x) * kHgTrainRays;
+  {
+    for (int i = tid; i < kHgW * 2 * kHgLevels; i += kHgTrainThreads)
+      sw[(i >> 5) * kHgLdf + (i & 31)] = __ldg(mlp + (i >> 5) * kHgCode + (i & 31));
+    int src = kHgW * kHgCode + kHgW, dst = kHgW * kHgLdf;
+    for (int l = 1; l < H; ++l) {
+      for (int i = tid; i < kHgW * kHgW; i += kHgTrainThreads)
+        sw[dst + (i >> 6) * kHgLdw + (i & 63)] = __ldg(mlp + src + i);
+      src += kHgW * kHgW + kHgW;
+      dst += kHgW * kHgLdw;
+    }
+    for (int i = tid; i < 2 * kHgW; i += kHgTrainThreads) sw[dst + i] = __ldg(mlp + src + i);
   }
-  const float* wo = sw + off;
+  __syncthreads();
+  const int r = tid & 31, t = tid >> 5;
+  const int64_t row = row0 + r;
+  const bool valid = row < M;
+  const float* wo = sw + kHgW * kHgLdf + (H - 1) * kHgW * kHgLdw;
   const float2 d = valid ? dz[row] : make_float2(0.f, 0.f);
-  for (int k = t; k < kHgW; k += kHgTrainT) dh[k] = d.x * wo[k] + d.y * wo[kHgW + k];
-  __syncwarp();
+  float* dh = bufA;
+  float* dn = bufB;
+  for (int k = t; k < kHgW; k += kHgTrainT) dh[k * kHgLda + r] = d.x * wo[k] + d.y * wo[kHgW + k];
+  const int tr = tid & 15, tn = tid >> 4;
   for (int l = H - 1; l >= 0; --l) {
+    // the thread that wrote (or, below, will have passed a barrier after) dh
+    // masks it by its layer's ReLU
     const float* h = acts + static_cast<int64_t>(l) * kHgW * M + row;
     float* dp = dpre + static_cast<int64_t>(l) * kHgW * M + row;
-    for (int k = t; k < kHgW; k += kHgTrainT) {
-      const float v = valid && h[k * M] > 0.f ? dh[k] : 0.f;
-      dh[k] = v;
+#pragma unroll
+    for (int q = 0; q < kHgW / kHgTrainT; ++q) {
+      const int k = t + kHgTrainT * q;
+      const float v = valid && h[k * M] > 0.f ? dh[k * kHgLda + r] : 0.f;
+      dh[k * kHgLda + r] = v;
       if (valid) dp[k * M] = v;
     }
-    __syncwarp();
-    const int K = l == 0 ? 2 * 16 : kHgW;  // layer 1: only the hash features need a gradient
-    const int ldw = l == 0 ? kHgCode : kHgW;
-    const float* w = sw + woff[l];
-    float sacc[kHgW / kHgTrainT];
-#pragma unroll
-    for (int q = 0; q < kHgW / kHgTrainT; ++q) sacc[q] = 0.f;
-    for (int n = 0; n < kHgW; ++n) {
-      const float dv = dh[n];
-      const float* wr = w + n * ldw + t;
-#pragma unroll
-      for (int q = 0; q < kHgW / kHgTrainT; ++q)
-        if (t + kHgTrainT * q < K) sacc[q] = fmaf(dv, wr[kHgTrainT * q], sacc[q]);
+    __syncthreads();
+    float acc[2][4];
+    if (l > 0) {
+      hg_tile(dh, sw + kHgW * kHgLdf + (l - 1) * kHgW * kHgLdw, kHgLdw, kHgW, tr, tn, acc);
+    } else if (tn < 2 * kHgLevels / 4) {  // layer 1: only the hash features need a gradient
+      hg_tile(dh, sw, kHgLdf, kHgW, tr, tn, acc);
     }
+    if (l > 0 || tn < 2 * kHgLevels / 4) {
 #pragma unroll
-    for (int q = 0; q < kHgW / kHgTrainT; ++q)
-      if (t + kHgTrainT * q < K) dn[t + kHgTrainT * q] = sacc[q];
-    __syncwarp();
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<float2*>(dn + (4 * tn + j) * kHgLda + 2 * tr) =
+            make_float2(acc[0][j], acc[1][j]);
+    }
+    __syncthreads();
     float* tmp = dh;
     dh = dn;
     dn = tmp;
   }
   if (!valid) return;
-  // dh holds dL/d(hash features) [32]: this thread scatters levels t,
-  // t + kHgTrainT, ...
-  const float x = box01(rays.p[0][row]), y = box01(rays.p[1][row]), z = box01(rays.p[2][row]);
+  // dh holds dL/d(hash features) [32]: this thread scatters levels t and t + 8
+  const float x = box01(__ldg(rays.p[0] + row)), y = box01(__ldg(rays.p[1] + row)),
+              z = box01(__ldg(rays.p[2] + row));
+#pragma unroll
   for (int j = 0; j < kHgLevels / kHgTrainT; ++j) {
     const int l = t + kHgTrainT * j;
     const int n = g.res[l];
@@ -548,7 +657,8 @@ __global__ void __launch_bounds__(kHgTrainThreads)
     const float wx = ux - static_cast<float>(ix);
     const float wy = uy - static_cast<float>(iy);
     const float wz = uz - static_cast<float>(iz);
-    const float g0 = dh[2 * l], g1 = dh[2 * l + 1];
+    const float g0 = dh[(2 * l) * kHgLda + r], g1 = dh[(2 * l + 1) * kHgLda + r];
+#pragma unroll
     for (int c = 0; c < 8; ++c) {
       const float w = ((c & 1) ? wx : 1.f - wx) * (((c >> 1) & 1) ? wy : 1.f - wy) *
                       ((c >> 2) ? wz : 1.f - wz);
@@ -570,8 +680,8 @@ __global__ void __launch_bounds__(kHgTrainThreads)
 // in order.
 __global__ void __launch_bounds__(256)
 hg_outer_tiled_kernel(const HgOuterJobs jobs, int64_t B, int64_t per_split) {
-  __shared__ float sP[32][65];
-  __shared__ float sA[32][65];
+  constexpr int kLd = 68;  // 16-byte rows
+  __shared__ __align__(16) float sP[32 * kLd], sA[32 * kLd];
   const HgOuterJob& jb = jobs.job[blockIdx.y];
   const float* __restrict__ P = jb.P;
   const float* __restrict__ A = jb.A;
@@ -583,23 +693,32 @@ hg_outer_tiled_kernel(const HgOuterJobs jobs, int64_t B, int64_t per_split) {
   const int64_t r1 = r0 + per_split < B ? r0 + per_split : B;
   float acc[4][4] = {};
   float bs[4] = {0.f, 0.f, 0.f, 0.f};
+  // the next slice is on its way while this one is summed
+  const int lr = tid & 31, lc = tid >> 5;  // a warp reads 32 rays of one feature
+  float np_[8], na_[8];
+  auto load = [&](int64_t rb) {
+    const int64_t r = rb + lr;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int c = lc + 8 * j;
+      np_[j] = r < r1 && c < np ? P[r * prs + c * pcs] : 0.f;
+      na_[j] = r < r1 && c < na ? A[r * ars + c * acs] : 0.f;
+    }
+  };
+  load(r0);
   for (int64_t rb = r0; rb < r1; rb += 32) {
-    for (int i = tid; i < 32 * 64; i += 256) {
-      const int rr = i & 31, c = i >> 5;  // a warp reads 32 rays of one feature
-      const int64_t r = rb + rr;
-      const bool ok = r < r1;
-      sP[rr][c] = ok && c < np ? P[r * prs + c * pcs] : 0.f;
-      sA[rr][c] = ok && c < na ? A[r * ars + c * acs] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      sP[lr * kLd + lc + 8 * j] = np_[j];
+      sA[lr * kLd + lc + 8 * j] = na_[j];
     }
     __syncthreads();
-#pragma unroll 4
+    if (rb + 32 < r1) load(rb + 32);
+#pragma unroll 8
     for (int rr = 0; rr < 32; ++rr) {
-      float pv[4], av[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        pv[i] = sP[rr][4 * tn + i];
-        av[i] = sA[rr][4 * tk + i];
-      }
+      const float4 p4 = *reinterpret_cast<const float4*>(sP + rr * kLd + 4 * tn);
+      const float4 a4 = *reinterpret_cast<const float4*>(sA + rr * kLd + 4 * tk);
+      const float pv[4] = {p4.x, p4.y, p4.z, p4.w}, av[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         bs[i] += pv[i];
@@ -713,37 +832,34 @@ int hashgrid_tc_blocks_per_sm(int H) {
 cudaError_t launch_hashgrid_f32(const HashGridParams& g, const float2* table, const float* mlp,
                                 int H, RaySoA rays, int64_t M, HeadOut out, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
-  if (H < 1 || H > 4) return cudaErrorInvalidValue;
-  const int n_mlp = kHgW * kHgCode + kHgW + (H - 1) * (kHgW * kHgW + kHgW) + 2 * kHgW + 2;
-  const size_t smem = (((n_mlp + 3) & ~3) + 2 * kHgF32Rays * kHgLd) * sizeof(float);
+  if (H < 1 || H > 4 || (reinterpret_cast<uintptr_t>(table) & 15u) != 0)
+    return cudaErrorInvalidValue;
+  const int smem = (hg_wt_floats(H) + kHgW * kHgF32Ld) * static_cast<int>(sizeof(float));
   cudaError_t e = cudaFuncSetAttribute(hashgrid_f32_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return e;
   const int64_t blocks = (M + kHgF32Rays - 1) / kHgF32Rays;
-  hashgrid_f32_kernel<<<static_cast<unsigned>(blocks), kHgF32Rays, smem, s>>>(
-      g, table, mlp, H, rays, M, out);
+  const int64_t grid = blocks < kHgF32Ctas * sms ? blocks : kHgF32Ctas * sms;
+  hashgrid_f32_kernel<<<static_cast<unsigned>(grid), kHgF32Threads, smem, s>>>(g, table, mlp, H,
+                                                                               rays, M, out);
   return cudaGetLastError();
 }
-
-namespace {
-size_t hg_f32_smem(int H) {
-  const int n_mlp = kHgW * kHgCode + kHgW + (H - 1) * (kHgW * kHgW + kHgW) + 2 * kHgW + 2;
-  return (((n_mlp + 3) & ~3) + 2 * kHgF32Rays * kHgLd) * sizeof(float);
-}
-}  // namespace
 
 cudaError_t launch_hg_train_fwd(const HashGridParams& g, const float2* table, const float* mlp,
                                 int H, RaySoA rays, int64_t B, float* code, float* acts,
                                 float2* z, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
-  if (H < 1 || H > 4) return cudaErrorInvalidValue;
-  const size_t smem = (((hg_train_wfloats(H) + 3) & ~3) + 2 * kHgF32Rays * kHgLd) * sizeof(float);
+  if (H < 1 || H > 4 || (reinterpret_cast<uintptr_t>(table) & 15u) != 0)
+    return cudaErrorInvalidValue;
+  const int smem = (hg_wt_floats(H) + 2 * kHgW * kHgLda) * static_cast<int>(sizeof(float));
   cudaError_t e = cudaFuncSetAttribute(hg_train_fwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (B + kHgF32Rays - 1) / kHgF32Rays;
+  const int64_t blocks = (B + kHgTrainRays - 1) / kHgTrainRays;
   hg_train_fwd_kernel<<<static_cast<unsigned>(blocks), kHgTrainThreads, smem, s>>>(
       g, table, mlp, H, rays, B, code, acts, z);
   return cudaGetLastError();
@@ -755,12 +871,11 @@ cudaError_t launch_hg_train_bwd(const HashGridParams& g, const float* mlp, int H
   if (B <= 0) return cudaSuccess;
   if (H < 1 || H > 4) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(grad_table) & 7u) != 0) return cudaErrorInvalidValue;
-  const size_t smem = hg_f32_smem(H);
+  const int smem = (hg_bwd_floats(H) + 2 * kHgW * kHgLda) * static_cast<int>(sizeof(float));
   cudaError_t e = cudaFuncSetAttribute(hg_train_bwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (B + kHgF32Rays - 1) / kHgF32Rays;
+  const int64_t blocks = (B + kHgTrainRays - 1) / kHgTrainRays;
   hg_train_bwd_kernel<<<static_cast<unsigned>(blocks), kHgTrainThreads, smem, s>>>(
       g, mlp, H, rays, B, acts, dz, dpre, grad_table);
   return cudaGetLastError();
