@@ -231,6 +231,8 @@ constexpr float kLossClamp = 4.0f;
 constexpr float kLossLambda = 0.3f;
 constexpr float kAdamB1 = 0.9f, kAdamB2 = 0.999f, kAdamEps = 1e-8f;
 
+ddf_status ensure_reduce_stream(ddf_s* h);
+
 // hash-grid field (hashgrid_api.cpp)
 // Level layout; even_offsets pads each level to start on an even entry.
 ddf::HashGridParams hg_layout(int64_t* entries, bool even_offsets);

@@ -284,6 +284,14 @@ cudaError_t launch_head_train(const __nv_bfloat16* H, int M, int W, const float*
 cudaError_t launch_loss(const float2* z, const float* t_tgt, const uint8_t* y, int64_t B,
                         unsigned* nhit, float clamp, float lam, float2* dz, float* part,
                         float* loss_out, cudaStream_t s);
+// Its three parts, for a caller that runs them on different streams: the
+// number of hits; the loss terms (summed per block into part) and dL/dz, from
+// that number; the sum of the part.
+cudaError_t launch_count_hits(const uint8_t* y, int64_t B, unsigned* nhit, cudaStream_t s);
+cudaError_t launch_loss_dz(const float2* z, const float* t_tgt, const uint8_t* y, int64_t B,
+                           const unsigned* nhit, float clamp, float lam, float2* dz, float* part,
+                           cudaStream_t s);
+cudaError_t launch_loss_sum(const float* part, int64_t B, float* loss_out, cudaStream_t s);
 // One pass over H [M x W]: dpre = bf16((dz wo) where H > 0), and per split
 // of rows part [splits x (3 W + 4)]: partials of dz0 H, dz1 H, of dpre's
 // column sums and of dz0, dz1 (each summed over the split's rows in order;

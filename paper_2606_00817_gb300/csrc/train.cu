@@ -134,12 +134,26 @@ __global__ void sdf_loss_kernel(const float2* __restrict__ z, const float* __res
   }
 }
 
-__global__ void sum_partials_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float t = 0.f;
-    for (int i = 0; i < n; ++i) t += part[i];
-    *out = t;
+constexpr int kSumThreads = 256;
+
+// The n partial sums added in order by one thread, from shared memory: with a
+// dependent global load each, 256 of them took 6.7 us.
+__global__ void __launch_bounds__(kSumThreads)
+sum_partials_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
+  __shared__ float s[kSumThreads];
+  float t = 0.f;
+  for (int base = 0; base < n; base += kSumThreads) {
+    const int i = base + threadIdx.x;
+    s[threadIdx.x] = i < n ? part[i] : 0.f;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const int m = min(n - base, kSumThreads);
+#pragma unroll 16
+      for (int k = 0; k < m; ++k) t += s[k];
+    }
+    __syncthreads();
   }
+  if (threadIdx.x == 0) *out = t;
 }
 
 // The head's backward in one pass over the last activation H [M x W] (bf16):
@@ -255,6 +269,8 @@ __device__ __forceinline__ void add4(float4& a, const float4 b) {
   a.w += b.w;
 }
 
+constexpr int kRedBatch = 8;  // 16-byte loads in flight a thread
+
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant__ GradReduce g) {
   const int b = blockIdx.x;
   if (b < g.blk0[g.nsplit]) {
@@ -263,26 +279,42 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant_
     const RedSplit& a = g.split[j];
     const int64_t e0 = 4 * (static_cast<int64_t>(b - g.blk0[j]) * blockDim.x + threadIdx.x);
     const int64_t total = static_cast<int64_t>(a.rows) * a.cols;
-    if (e0 >= total) return;
     if (a.vec) {
+      if (e0 >= total) return;
       const int r = static_cast<int>(e0 / a.cols);
       const int c = static_cast<int>(e0 - static_cast<int64_t>(r) * a.cols);
       const float* src = a.part + static_cast<int64_t>(r) * a.ldp + c;
       float* dst = a.out + static_cast<int64_t>(r) * a.ldo + c;  // cols, ldp, ldo, split_stride multiples of 4; 16-byte aligned
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int q = 0; q < a.S; ++q) add4(acc, *reinterpret_cast<const float4*>(src + q * a.split_stride));
+      for (int q0 = 0; q0 < a.S; q0 += kRedBatch) {  // loads in flight together, added in order
+        float4 v[kRedBatch];
+#pragma unroll
+        for (int j = 0; j < kRedBatch; ++j)
+          if (q0 + j < a.S) v[j] = *reinterpret_cast<const float4*>(src + (q0 + j) * a.split_stride);
+#pragma unroll
+        for (int j = 0; j < kRedBatch; ++j)
+          if (q0 + j < a.S) add4(acc, v[j]);
+      }
       *reinterpret_cast<float4*>(dst) = acc;
       return;
     }
-    for (int k = 0; k < 4 && e0 + k < total; ++k) {  // the 4 elements may span rows
-      const int rk = static_cast<int>((e0 + k) / a.cols);
-      const int ck = static_cast<int>(e0 + k - static_cast<int64_t>(rk) * a.cols);
-      const float* sk = a.part + static_cast<int64_t>(rk) * a.ldp + ck;
-      float acc = 0.f;
-      for (int q = 0; q < a.S; ++q) acc += sk[q * a.split_stride];
-      a.out[static_cast<int64_t>(rk) * a.ldo + ck] = acc;
+    // rows of any length: one element a thread
+    const int64_t e = static_cast<int64_t>(b - g.blk0[j]) * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int r = static_cast<int>(e / a.cols);
+    const int c = static_cast<int>(e - static_cast<int64_t>(r) * a.cols);
+    const float* src = a.part + static_cast<int64_t>(r) * a.ldp + c;
+    float acc = 0.f;
+    for (int q0 = 0; q0 < a.S; q0 += 2 * kRedBatch) {
+      float v[2 * kRedBatch];
+#pragma unroll
+      for (int j = 0; j < 2 * kRedBatch; ++j)
+        if (q0 + j < a.S) v[j] = src[(q0 + j) * a.split_stride];
+#pragma unroll
+      for (int j = 0; j < 2 * kRedBatch; ++j)
+        if (q0 + j < a.S) acc += v[j];
     }
+    a.out[static_cast<int64_t>(r) * a.ldo + c] = acc;
     return;
   }
   const RedCols& cs = g.cols;
@@ -380,43 +412,68 @@ __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, 
   }
 }
 
+// a / b correctly rounded, given r = 1 / b correctly rounded: Markstein's
+// division (P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", IBM J. Res. Dev. 34, 1990, theorem 7.2): the product
+// a r corrected once by its exact remainder. Where the remainder falls below
+// the smallest normal number (|a| under about 1e-30) the quotient may be off in
+// its last places.
+__device__ __forceinline__ float div_by(float a, float b, float r) {
+  const float q = a * r;
+  return fmaf(fmaf(-q, b, a), r, q);
+}
+
 // Adam over the level tables of a hash-grid field (entry i of the blob is
 // the feature pair 2 i, 2 i + 1) and, in the same pass, their bf16x2 query
 // copy: source entry i of level l goes to word i - from.offset[l] +
 // to.offset[l] (f0 in the low half). The arithmetic of adam_kernel, element
 // by element; two entries (one float4 of each array) per thread when vec.
-__global__ void hg_adam_pack_kernel(float* __restrict__ w, const float* __restrict__ g,
-                                    float* __restrict__ m, float* __restrict__ v, int64_t entries,
-                                    float lr, float b1, float b2, float eps, float bc1, float bc2,
-                                    HashGridParams from, HashGridParams to,
-                                    uint32_t* __restrict__ dst, int vec) {
+// With three general divisions an element it was bound by arithmetic (88 us,
+// 79 % of the issue slots, DRAM at 47 %); the two by the bias corrections, the
+// same for every element, take 3 instructions each. The moments and the
+// gradient are read (and the moments written) as streams, which leaves the
+// tables in L2 for the next step's gathers. 6.5 M entries: 63 us, 392 MB of
+// traffic at 6.2 TB/s.
+__global__ void __launch_bounds__(256)
+hg_adam_pack_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
+                    float* __restrict__ v, int64_t entries, float lr, float b1, float b2,
+                    float eps, float bc1, float bc2, const __grid_constant__ HashGridParams from,
+                    const __grid_constant__ HashGridParams to, uint32_t* __restrict__ dst,
+                    int vec) {
   const int64_t e0 = 2 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (e0 >= entries) return;
-  auto word = [&](int64_t e) {
-    int l = 0;
+  auto word = [&](uint32_t e) {  // entries < 2^32
+    uint32_t d = to.offset[0] - from.offset[0];
 #pragma unroll
-    for (int k = 1; k < 16; ++k) l += e >= from.offset[k] ? 1 : 0;
-    return e - from.offset[l] + to.offset[l];
+    for (int k = 1; k < 16; ++k)
+      if (e >= from.offset[k]) d = to.offset[k] - from.offset[k];
+    return e + d;
   };
   auto pack = [](float lo, float hi) {
     __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&b);
   };
+  const float r1 = 1.f / bc1, r2 = 1.f / bc2;
+  auto elem = [&](float we, float ge, float& me, float& ve) {  // as adam_elem
+    me = fmaf(b1, me, (1.f - b1) * ge);
+    ve = fmaf(b2, ve, (1.f - b2) * ge * ge);
+    return we - lr * div_by(me, bc1, r1) / (sqrtf(div_by(ve, bc2, r2)) + eps);
+  };
   const int64_t i4 = 2 * e0;
   if (vec && e0 + 2 <= entries) {
+    const float4 G = __ldcs(reinterpret_cast<const float4*>(g + i4));
+    float4 M = __ldcs(reinterpret_cast<const float4*>(m + i4));
+    float4 V = __ldcs(reinterpret_cast<const float4*>(v + i4));
     float4 W = *reinterpret_cast<const float4*>(w + i4);
-    const float4 G = *reinterpret_cast<const float4*>(g + i4);
-    float4 M = *reinterpret_cast<const float4*>(m + i4);
-    float4 V = *reinterpret_cast<const float4*>(v + i4);
-    W.x = adam_elem(W.x, G.x, M.x, V.x, lr, b1, b2, eps, bc1, bc2);
-    W.y = adam_elem(W.y, G.y, M.y, V.y, lr, b1, b2, eps, bc1, bc2);
-    W.z = adam_elem(W.z, G.z, M.z, V.z, lr, b1, b2, eps, bc1, bc2);
-    W.w = adam_elem(W.w, G.w, M.w, V.w, lr, b1, b2, eps, bc1, bc2);
-    *reinterpret_cast<float4*>(m + i4) = M;
-    *reinterpret_cast<float4*>(v + i4) = V;
+    W.x = elem(W.x, G.x, M.x, V.x);
+    W.y = elem(W.y, G.y, M.y, V.y);
+    W.z = elem(W.z, G.z, M.z, V.z);
+    W.w = elem(W.w, G.w, M.w, V.w);
+    __stcs(reinterpret_cast<float4*>(m + i4), M);
+    __stcs(reinterpret_cast<float4*>(v + i4), V);
     *reinterpret_cast<float4*>(w + i4) = W;
-    dst[word(e0)] = pack(W.x, W.y);
-    dst[word(e0 + 1)] = pack(W.z, W.w);
+    dst[word(static_cast<uint32_t>(e0))] = pack(W.x, W.y);
+    dst[word(static_cast<uint32_t>(e0) + 1)] = pack(W.z, W.w);
     return;
   }
   for (int64_t e = e0; e < e0 + 2 && e < entries; ++e) {
@@ -424,12 +481,12 @@ __global__ void hg_adam_pack_kernel(float* __restrict__ w, const float* __restri
     for (int f = 0; f < 2; ++f) {
       const int64_t i = 2 * e + f;
       float mi = m[i], vi = v[i];
-      nw[f] = adam_elem(w[i], g[i], mi, vi, lr, b1, b2, eps, bc1, bc2);
+      nw[f] = elem(w[i], g[i], mi, vi);
       w[i] = nw[f];
       m[i] = mi;
       v[i] = vi;
     }
-    dst[word(e)] = pack(nw[0], nw[1]);
+    dst[word(static_cast<uint32_t>(e))] = pack(nw[0], nw[1]);
   }
 }
 
@@ -597,23 +654,41 @@ cudaError_t launch_head_sum(const float2* part, int nparts, int64_t M, const flo
   return cudaGetLastError();
 }
 
+cudaError_t launch_count_hits(const uint8_t* y, int64_t B, unsigned* nhit, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(nhit, 0, sizeof(unsigned), s);
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = (B + 255) / 256;
+  count_hits_kernel<<<static_cast<unsigned>(blocks < 256 ? blocks : 256), 256, 0, s>>>(y, B, nhit);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_loss_dz(const float2* z, const float* t_tgt, const uint8_t* y, int64_t B,
+                           const unsigned* nhit, float clamp, float lam, float2* dz, float* part,
+                           cudaStream_t s) {
+  loss_dz_kernel<<<static_cast<unsigned>((B + 255) / 256), 256, 0, s>>>(z, t_tgt, y, B, nhit,
+                                                                         clamp, lam, dz, part);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_loss_sum(const float* part, int64_t B, float* loss_out, cudaStream_t s) {
+  if (loss_out == nullptr) return cudaSuccess;
+  sum_partials_kernel<<<1, kSumThreads, 0, s>>>(part, static_cast<int>((B + 255) / 256), loss_out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_loss(const float2* z, const float* t_tgt, const uint8_t* y, int64_t B,
                         unsigned* nhit, float clamp, float lam, float2* dz, float* part,
                         float* loss_out, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(nhit, 0, sizeof(unsigned), s);
-  if (e != cudaSuccess) return e;
-  count_hits_kernel<<<256, 256, 0, s>>>(y, B, nhit);
-  const int blocks = static_cast<int>((B + 255) / 256);
-  loss_dz_kernel<<<blocks, 256, 0, s>>>(z, t_tgt, y, B, nhit, clamp, lam, dz, part);
-  if (loss_out != nullptr) sum_partials_kernel<<<1, 32, 0, s>>>(part, blocks, loss_out);
-  return cudaGetLastError();
+  cudaError_t e = launch_count_hits(y, B, nhit, s);
+  if (e == cudaSuccess) e = launch_loss_dz(z, t_tgt, y, B, nhit, clamp, lam, dz, part, s);
+  return e != cudaSuccess ? e : launch_loss_sum(part, B, loss_out, s);
 }
 
 cudaError_t launch_sdf_loss(const float2* z, const float* s_tgt, int64_t B, float2* dz,
                             float* part, float* loss_out, cudaStream_t s) {
   const int blocks = static_cast<int>((B + 255) / 256);
   sdf_loss_kernel<<<blocks, 256, 0, s>>>(z, s_tgt, B, dz, part);
-  if (loss_out != nullptr) sum_partials_kernel<<<1, 32, 0, s>>>(part, blocks, loss_out);
+  if (loss_out != nullptr) sum_partials_kernel<<<1, kSumThreads, 0, s>>>(part, blocks, loss_out);
   return cudaGetLastError();
 }
 
@@ -639,7 +714,8 @@ cudaError_t launch_grad_reduce(const GradReduce& g0, cudaStream_t s) {
       return cudaErrorInvalidValue;
     a.vec = a.cols % 4 == 0 && a.ldp % 4 == 0 && a.ldo % 4 == 0 && a.split_stride % 4 == 0 &&
             al16(a.part) && al16(a.out);
-    const int64_t nb = (static_cast<int64_t>(a.rows) * a.cols + 1023) / 1024;
+    const int64_t per = a.vec ? 1024 : 256;  // elements a block
+    const int64_t nb = (static_cast<int64_t>(a.rows) * a.cols + per - 1) / per;
     if (g.blk0[j] + nb > (1ll << 30)) return cudaErrorInvalidValue;
     g.blk0[j + 1] = g.blk0[j] + static_cast<int>(nb);
   }

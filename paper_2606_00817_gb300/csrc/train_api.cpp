@@ -21,6 +21,31 @@
 #include "handle.h"
 #include "kernels.h"
 
+namespace ddfi {
+
+// The side stream of a training step (gradient reductions, and what else need
+// not hold up the main stream) and its events, made on first use.
+ddf_status ensure_reduce_stream(ddf_s* h) {
+  if (h->s_red != nullptr) return DDF_OK;
+  for (int b = 0; b < 2; ++b) {
+    if (h->ev_gemm[b] == nullptr)
+      DDF_CK(cudaEventCreateWithFlags(&h->ev_gemm[b], cudaEventDisableTiming));
+    if (h->ev_red[b] == nullptr)
+      DDF_CK(cudaEventCreateWithFlags(&h->ev_red[b], cudaEventDisableTiming));
+  }
+  if (h->ev_join == nullptr) DDF_CK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
+  // a hash grid's side kernels are small and run beside an Adam pass of many
+  // thousand blocks, behind which they would queue without a priority; beside
+  // the persistent GEMMs of a layered field they keep the usual one
+  int least = 0, greatest = 0;
+  DDF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+  DDF_CK(cudaStreamCreateWithPriority(&h->s_red, cudaStreamNonBlocking,
+                                      h->cfg.kind == DDF_KIND_HASHGRID ? greatest : least));
+  return DDF_OK;
+}
+
+}  // namespace ddfi
+
 using namespace ddfi;
 
 namespace {
@@ -342,21 +367,6 @@ ddf_status forward_keep(ddf_s* h, const float* const rays[6], int B, cudaStream_
     DDF_CK(ddf::launch_head_sum(h->tr_hz, train_head_parts(W), B, h->head_b, h->tr_z, st));
   else
     DDF_CK(ddf::launch_head_train(bf(h->tr_h[H - 1]), B, W, h->head_w, h->head_b, h->tr_z, st));
-  return DDF_OK;
-}
-
-// The stream the layers' gradient reductions run on and its events, made on
-// first use.
-ddf_status ensure_reduce_stream(ddf_s* h) {
-  if (h->s_red != nullptr) return DDF_OK;
-  for (int b = 0; b < 2; ++b) {
-    if (h->ev_gemm[b] == nullptr)
-      DDF_CK(cudaEventCreateWithFlags(&h->ev_gemm[b], cudaEventDisableTiming));
-    if (h->ev_red[b] == nullptr)
-      DDF_CK(cudaEventCreateWithFlags(&h->ev_red[b], cudaEventDisableTiming));
-  }
-  if (h->ev_join == nullptr) DDF_CK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
-  DDF_CK(cudaStreamCreateWithFlags(&h->s_red, cudaStreamNonBlocking));
   return DDF_OK;
 }
 
