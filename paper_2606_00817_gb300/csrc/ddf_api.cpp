@@ -119,6 +119,7 @@ void release_weight_buffers(ddf_s* h) {
   for (__nv_bfloat16* q : h->wp) dev_free(h, q);
   for (uint8_t* q : h->wq) dev_free(h, q);
   h->wb.clear();
+  h->tmBig.clear();
   h->wcal.clear();
   h->wp.clear();
   h->wq.clear();
@@ -347,8 +348,19 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
     DDF_CK(ddf::launch_tc_narrow(p, rays, out, W, h->num_sms, st));
     return DDF_OK;
   }
+  // the tiles in force: those set, or by the batch where none were (kPairRows)
+  const bool big = h->tile_auto && !h->tmBig.empty() && m >= kPairRows;
+  ddf::TcTile tile_h = h->tile, tile_1 = h->tile_first;
+  if (big) {
+    tile_h = ddf::TcTile{256, 4, true, true, false};
+    if (h->cfg.kind == DDF_KIND_RAY && H > 1 && ddf::tc_layer1_supported(h->cfg.octaves, W))
+      tile_1 = ddf::TcTile{256, 8, false, true, true};
+    else if (H > 1)
+      tile_1 = tile_h;
+  }
+  const std::vector<CUtensorMap>& tmB = big ? h->tmBig : h->tmB;
   // layer 1 may build the encoding itself (ddf_set_tile checked the shape)
-  const bool fused1 = h->tile_first.fused && h->cfg.kind == DDF_KIND_RAY;
+  const bool fused1 = tile_1.fused && h->cfg.kind == DDF_KIND_RAY;
   if (!fused1) {
     ProfScope ps(h, kProfEncode, st);
     if (h->cfg.kind == DDF_KIND_SDF)  // points in rays.p[0..2]
@@ -379,13 +391,13 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
     p.status = h->status_dev;
     p.timeout_ns = h->timeout_ns;
     ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
-    const ddf::TcTile& t = l == 0 ? h->tile_first : h->tile;
+    const ddf::TcTile& t = l == 0 ? tile_1 : tile_h;
     if (l == 0 && fused1) {
       CUtensorMap tmO;  // the layer's output, written by TMA stores of 32-row boxes
       if (!make_tmap(&tmO, p.out, out_fp8, W, m, static_cast<uint64_t>(W) * (out_fp8 ? 1 : 2), 32))
         return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an output map");
       const int grid = static_cast<int>(std::min<int64_t>((m + 127) / 128, h->num_sms));
-      DDF_CK(ddf::launch_tc_layer1(t.epi_warps, out_fp8, h->tmB[0], tmO, rays, h->cfg.octaves, p,
+      DDF_CK(ddf::launch_tc_layer1(t.epi_warps, out_fp8, tmB[0], tmO, rays, h->cfg.octaves, p,
                                    grid, st));
       continue;
     }
@@ -403,18 +415,39 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
           return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an output map");
         p.tma_out = 1;
       }
-      DDF_CK(ddf::launch_tc_gemm_pair(in_fp8, out_fp8, t.staged, t.epi_warps, tmA, h->tmB[l], p,
+      DDF_CK(ddf::launch_tc_gemm_pair(in_fp8, out_fp8, t.staged, t.epi_warps, tmA, tmB[l], p,
                                       clusters, st, tma_out ? &tmO : nullptr));
     } else {
       const int64_t tiles = ((m + 127) / 128) * static_cast<int64_t>(W / t.bn);
       const int grid = static_cast<int>(std::min<int64_t>(tiles, h->num_sms));
-      DDF_CK(ddf::launch_tc_gemm(t, in_fp8, out_fp8, tmA, h->tmB[l], p, grid, st));
+      DDF_CK(ddf::launch_tc_gemm(t, in_fp8, out_fp8, tmA, tmB[l], p, grid, st));
     }
   }
   ProfScope ps(h, kProfHead, st);
-  const ddf::TcTile& tl = H == 1 ? h->tile_first : h->tile;  // the last layer writes the partials
+  const ddf::TcTile& tl = H == 1 ? tile_1 : tile_h;  // the last layer writes the partials
   const int nparts = (tl.pair ? W / 256 : W / tl.bn) * (tl.epi_warps / 4);
   DDF_CK(ddf::launch_finish_heads(h->ws_part, nparts, m, h->head_b, out, st));
+  return DDF_OK;
+}
+
+// The weight maps of the tiles large batches take (kPairRows), once the weights
+// are loaded; none where those tiles do not exist.
+ddf_status build_big_maps(ddf_s* h) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  h->tmBig.clear();
+  if (h->cfg.precision == DDF_FP32 || W % 256 != 0 || h->pair_clusters <= 0) return DDF_OK;
+  std::vector<CUtensorMap> maps(H);
+  for (int l = 0; l < H; ++l) {
+    const bool whole = l == 0 && (H == 1 || (h->cfg.kind == DDF_KIND_RAY &&
+                                             ddf::tc_layer1_supported(h->cfg.octaves, W)));
+    const uint32_t box = whole ? 256u : 128u;  // layer 1 fused (or alone): 256 rows
+    const int kp = l == 0 ? h->kp16 : W;
+    const bool ok = h->wb[l] != nullptr
+                        ? make_tmap(&maps[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2, box)
+                        : make_tmap(&maps[l], h->wq[l], true, W, W, W, box);
+    if (!ok) return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+  }
+  h->tmBig = maps;
   return DDF_OK;
 }
 
@@ -935,6 +968,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     release_weight_buffers(h);  // the next load allocates again from nothing
     return s;
   }
+  if (h->tmBig.empty() && (s = build_big_maps(h)) != DDF_OK) return s;
   DDF_CK(cudaMemcpy(h->d_blob, host_blob, need * sizeof(float), cudaMemcpyHostToDevice));
   size_t off = 0;
   for (int l = 0; l < H; ++l) {

@@ -39,6 +39,7 @@ struct ddf_s {
   // tiles were set by the caller or found faster by the autotuner
   bool narrow = false;
   bool tile_auto = true;
+  std::vector<CUtensorMap> tmBig;  // weight maps of the tiles that large batches take by themselves
   CUtensorMap* narrow_maps = nullptr;  // device: a launch does not carry 2 KB of maps
   int pair_clusters = 0;  // co-resident clusters of the CTA-pair kernel
   int num_sms = 0;
@@ -186,6 +187,15 @@ struct DeviceGuard {
     if (prev >= 0) cudaSetDevice(prev);
   }
 };
+
+// Rows from which a field whose tiles nobody set takes the staged CTA-pair tile
+// for its hidden layers and the fused layer 1 (the same bits as the default
+// tiles): at 1280 x 8, default against these tiles, bf16 8,192 rows 248 and 242
+// us, 12,000 rows 313 and 289, 140,000 rows 2,217 and 1,965; e4m3 8,192 rows 177
+// and 173, 16,384 rows 230 and 230, 140,000 rows 1,227 and 1,123; at 512 x 6,
+// 8,192 rows 77 and 84, 12,000 rows 100 and 95. Below, a 256 x 256 tile leaves
+// too many SMs idle.
+constexpr int64_t kPairRows = 10240;
 
 constexpr int kProfClasses = 4;
 enum ProfClass { kProfEncode = 0, kProfGemm = 1, kProfHead = 2, kProfFirst = 3 };
