@@ -120,6 +120,7 @@ void release_weight_buffers(ddf_s* h) {
   for (uint8_t* q : h->wq) dev_free(h, q);
   h->wb.clear();
   h->tmBig.clear();
+  h->tmSmall.clear();
   h->wcal.clear();
   h->wp.clear();
   h->wq.clear();
@@ -185,6 +186,12 @@ int max_partials(int W) { return (W / 128) * 2; }
 
 void clear_graphs(ddf_s* h);
 
+// Fields whose small batches run on the tiles of tc_small.cu (narrow ones have
+// their own kernel).
+bool small_batches(const ddf_s* h) {
+  return h->cfg.kind == DDF_KIND_RAY && h->cfg.precision != DDF_FP32 && !h->narrow;
+}
+
 ddf_status ensure_workspace(ddf_s* h, int64_t rows) {
   if (rows <= h->ws_rows || h->cfg.kind == DDF_KIND_HASHGRID) return DDF_OK;  // no workspace
   clear_graphs(h);  // cached graphs point at the old buffers
@@ -194,6 +201,8 @@ ddf_status ensure_workspace(ddf_s* h, int64_t rows) {
   dev_free(h, h->ws_part);
   h->ws_enc = h->ws_act[0] = h->ws_act[1] = nullptr;
   h->ws_part = nullptr;
+  h->ws_x = nullptr;
+  h->ws_x_rows = 0;
   h->ws_rows = 0;
   const int W = h->cfg.width;
   const bool f32 = h->cfg.precision == DDF_FP32;
@@ -204,8 +213,15 @@ ddf_status ensure_workspace(ddf_s* h, int64_t rows) {
   const size_t r = static_cast<size_t>(planes ? std::min(rows, h->f32_pass) : rows);
   ddf_status st;
   if ((st = dev_alloc(h, &h->ws_enc, r * (f32 ? h->kp32 : h->kp16) * elem)) != DDF_OK) return st;
-  for (int i = 0; i < 2; ++i)
-    if ((st = dev_alloc(h, &h->ws_act[i], r * W * elem)) != DDF_OK) return st;
+  // the buffer the last layer would write holds a small batch's FP32 activations
+  const int xi = (h->cfg.hidden_layers - 1) & 1;
+  const int64_t xr = small_batches(h) ? std::min(rows, small_rows(W, h->num_sms)) : 0;
+  for (int i = 0; i < 2; ++i) {
+    const size_t bytes = std::max(r * W * elem, i == xi ? static_cast<size_t>(xr) * W * 4 : 0);
+    if ((st = dev_alloc(h, &h->ws_act[i], bytes)) != DDF_OK) return st;
+  }
+  h->ws_x = xr > 0 ? static_cast<float*>(h->ws_act[xi]) : nullptr;
+  h->ws_x_rows = xr;
   if (!f32) {
     void* p;
     if ((st = dev_alloc(h, &p, static_cast<size_t>(rows) * max_partials(W) * sizeof(float2))) != DDF_OK)
@@ -329,6 +345,44 @@ ddf_status forward_f32(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cuda
   return DDF_OK;
 }
 
+// A few hundred rays through a wide bf16 or e4m3 field (tc_small.cu).
+ddf_status forward_small(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
+  {
+    ProfScope ps(h, kProfEncode, st);
+    DDF_CK(ddf::launch_small_encode(rays, m, h->cfg.octaves, h->kp16,
+                                    static_cast<__nv_bfloat16*>(h->ws_enc), st));
+  }
+  for (int l = 0; l < H; ++l) {
+    const bool in_fp8 = fp8 && l > 0, last = l == H - 1, out_fp8 = fp8 && !last;
+    ddf::TcGemmParams p{};
+    p.M = m;
+    p.N = W;
+    p.K = l == 0 ? h->kp16 : W;
+    p.bias = h->bias[l];
+    p.col_scale = in_fp8 ? h->colscale[l] : nullptr;
+    p.out_scale = out_fp8 ? 1.0f / h->act_scales[l] : 1.0f;
+    p.ldo = W;
+    if (last)
+      p.out_f32 = h->ws_x;
+    else
+      p.out = h->ws_act[l & 1];
+    p.status = h->status_dev;
+    p.timeout_ns = h->timeout_ns;
+    CUtensorMap tmA;
+    if (!make_tmap(&tmA, l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1], in_fp8, p.K, m,
+                   static_cast<uint64_t>(p.K) * (in_fp8 ? 1 : 2), 128))
+      return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
+    ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
+    DDF_CK(ddf::launch_small_layer(in_fp8, out_fp8, tmA, h->tmSmall[l], p, st));
+  }
+  ProfScope ps(h, kProfHead, st);
+  DDF_CK(ddf::launch_small_heads(h->ws_x, m, W, W % 256 == 0 ? 256 : 128, h->head_w, h->head_b,
+                                 out, st));
+  return DDF_OK;
+}
+
 ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
   const int W = h->cfg.width;
   const int H = h->cfg.hidden_layers;
@@ -348,6 +402,8 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
     DDF_CK(ddf::launch_tc_narrow(p, rays, out, W, h->num_sms, st));
     return DDF_OK;
   }
+  if (h->tile_auto && !h->tmSmall.empty() && m <= small_rows(W, h->num_sms) && m <= h->ws_x_rows)
+    return forward_small(h, rays, m, out, st);
   // the tiles in force: those set, or by the batch where none were (kPairRows)
   const bool big = h->tile_auto && !h->tmBig.empty() && m >= kPairRows;
   ddf::TcTile tile_h = h->tile, tile_1 = h->tile_first;
@@ -430,11 +486,23 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
   return DDF_OK;
 }
 
-// The weight maps of the tiles large batches take (kPairRows), once the weights
-// are loaded; none where those tiles do not exist.
-ddf_status build_big_maps(ddf_s* h) {
+// The weight maps of the tiles that batches take by their size (kPairRows,
+// small_rows), once the weights are loaded; none where those tiles do not exist.
+ddf_status build_size_maps(ddf_s* h) {
   const int W = h->cfg.width, H = h->cfg.hidden_layers;
   h->tmBig.clear();
+  h->tmSmall.clear();
+  if (small_batches(h)) {
+    std::vector<CUtensorMap> maps(H);
+    for (int l = 0; l < H; ++l) {
+      const int kp = l == 0 ? h->kp16 : W;
+      const bool ok = h->wb[l] != nullptr
+                          ? make_tmap(&maps[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2, 64)
+                          : make_tmap(&maps[l], h->wq[l], true, W, W, W, 64);
+      if (!ok) return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+    }
+    h->tmSmall = maps;
+  }
   if (h->cfg.precision == DDF_FP32 || W % 256 != 0 || h->pair_clusters <= 0) return DDF_OK;
   std::vector<CUtensorMap> maps(H);
   for (int l = 0; l < H; ++l) {
@@ -968,7 +1036,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     release_weight_buffers(h);  // the next load allocates again from nothing
     return s;
   }
-  if (h->tmBig.empty() && (s = build_big_maps(h)) != DDF_OK) return s;
+  if (h->tmBig.empty() && h->tmSmall.empty() && (s = build_size_maps(h)) != DDF_OK) return s;
   DDF_CK(cudaMemcpy(h->d_blob, host_blob, need * sizeof(float), cudaMemcpyHostToDevice));
   size_t off = 0;
   for (int l = 0; l < H; ++l) {
@@ -1670,6 +1738,15 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   void* act1 = p;
   p += up(static_cast<size_t>(rows) * W * act_elem);
   float2* part = f32 ? nullptr : reinterpret_cast<float2*>(p);
+  if (!f32) p += up(static_cast<size_t>(n) * max_partials(W) * sizeof(float2));
+  // the small-batch tiles' FP32 activations, where the scratch has room
+  const bool room = !f32 && small_batches(h) && n <= small_rows(W, h->num_sms) &&
+                    static_cast<size_t>(p - static_cast<uint8_t*>(ws)) +
+                            static_cast<size_t>(n) * W * sizeof(float) <= ws_bytes;
+  float* const save_x = h->ws_x;
+  const int64_t save_x_rows = h->ws_x_rows;
+  h->ws_x = room ? reinterpret_cast<float*>(p) : nullptr;
+  h->ws_x_rows = room ? n : 0;
 
   void* save_enc = h->ws_enc;
   void* save_act0 = h->ws_act[0];
@@ -1695,6 +1772,8 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   h->ws_act[0] = save_act0;
   h->ws_act[1] = save_act1;
   h->ws_part = save_part;
+  h->ws_x = save_x;
+  h->ws_x_rows = save_x_rows;
   h->ws_rows = save_rows;
   h->chunk = save_chunk;
   h->prof = save_prof;

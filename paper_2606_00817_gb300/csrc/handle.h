@@ -39,6 +39,7 @@ struct ddf_s {
   // tiles were set by the caller or found faster by the autotuner
   bool narrow = false;
   bool tile_auto = true;
+  std::vector<CUtensorMap> tmSmall;  // weight maps of the small-batch tile
   std::vector<CUtensorMap> tmBig;  // weight maps of the tiles that large batches take by themselves
   CUtensorMap* narrow_maps = nullptr;  // device: a launch does not carry 2 KB of maps
   int pair_clusters = 0;  // co-resident clusters of the CTA-pair kernel
@@ -86,6 +87,8 @@ struct ddf_s {
   void* ws_enc = nullptr;
   void* ws_act[2] = {nullptr, nullptr};
   float2* ws_part = nullptr;
+  float* ws_x = nullptr;  // small batches: the last layer's FP32 activations (one of ws_act)
+  int64_t ws_x_rows = 0;
 
   uint32_t* status_dev = nullptr;
 
@@ -196,6 +199,14 @@ struct DeviceGuard {
 // 8,192 rows 77 and 84, 12,000 rows 100 and 95. Below, a 256 x 256 tile leaves
 // too many SMs idle.
 constexpr int64_t kPairRows = 10240;
+
+// Rows up to which a field whose tiles nobody set runs its layers on 128 x 64
+// tiles (tc_small.cu): two waves of them. At 1280 x 8 bf16, these against the
+// default tiles: 800 rows 75 and 129 us, 1,000 rows 121 and 129, 1,920 rows 133
+// and 133; e4m3 1,920 rows 94 and 114; a third wave would lose.
+inline int64_t small_rows(int width, int num_sms) {
+  return 128 * (static_cast<int64_t>(2) * num_sms / (width / 64));
+}
 
 constexpr int kProfClasses = 4;
 enum ProfClass { kProfEncode = 0, kProfGemm = 1, kProfHead = 2, kProfFirst = 3 };

@@ -209,6 +209,18 @@ struct HeadOut {
 // From FP32 activations H [M x W] (FP32 path).
 cudaError_t launch_head_f32(const float* H, int M, int W, const float* wo, const float* bo,
                             HeadOut o, cudaStream_t s);
+// A wide field's layers for a small batch (tc_small.cu): 128 x 64 tiles,
+// launched with programmatic dependence on the kernel before. tmA as
+// launch_tc_gemm, tmB with boxes of 64 rows. Mode-0 output to p.out, or the
+// last layer's FP32 activations ReLU(y) [M x ldo] to p.out_f32 (32-byte
+// aligned) for launch_small_heads, which sums the head in chains over blocks of
+// `blk` columns. The same bits as the default tiles (blk = their bn).
+cudaError_t launch_small_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
+                               const CUtensorMap& tmB, const TcGemmParams& p, cudaStream_t s);
+cudaError_t launch_small_encode(const RaySoA& rays, int64_t M, int L, int ld, __nv_bfloat16* out,
+                                cudaStream_t s);
+cudaError_t launch_small_heads(const float* X, int M, int W, int blk, const float* wo,
+                               const float* bo, const HeadOut& o, cudaStream_t s);
 // From per-N-block partial dot products [nblk x M] (tensor-core path).
 cudaError_t launch_finish_heads(const float2* part, int nblk, int M, const float* bo, HeadOut o,
                                 cudaStream_t s);
