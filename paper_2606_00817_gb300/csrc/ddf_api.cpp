@@ -121,6 +121,7 @@ void release_weight_buffers(ddf_s* h) {
   h->wb.clear();
   h->tmBig.clear();
   h->tmSmall.clear();
+  h->tmTrace.clear();
   h->wcal.clear();
   h->wp.clear();
   h->wq.clear();
@@ -748,6 +749,53 @@ ddf_status ensure_trace_buffers(ddf_s* h, int64_t rows) {
   return DDF_OK;
 }
 
+// A trace by one persistent kernel (tc_trace.cu), for the fields and batches it
+// serves.
+ddf_status trace_in_one(ddf_s* h, const float* const rays[6], int n, int max_steps, float eps,
+                        float t_max, float* out_t, uint8_t* out_hit, int32_t* out_steps,
+                        cudaStream_t st) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  ddf_status s;
+  if (h->trc_queue == nullptr) {
+    void* q;
+    if ((s = dev_alloc(h, &q, sizeof(int))) != DDF_OK) return s;
+    h->trc_queue = static_cast<int*>(q);
+  }
+  if (static_cast<int>(h->tmTrace.size()) != H) {
+    std::vector<CUtensorMap> maps(H);
+    for (int l = 0; l < H; ++l) {
+      const int kp = l == 0 ? h->kp16 : W;
+      if (!make_tmap(&maps[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2, 128))
+        return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+    }
+    h->tmTrace = maps;
+  }
+  ddf::TraceMaps maps{};
+  ddf::TraceParams p{};
+  for (int c = 0; c < 6; ++c) p.rays.p[c] = rays[c];
+  p.n = n;
+  p.L = h->cfg.octaves;
+  p.H = H;
+  p.max_steps = max_steps;
+  p.eps = eps;
+  p.t_max = t_max;
+  for (int l = 0; l < H; ++l) {
+    maps.m[l] = h->tmTrace[l];
+    p.bias[l] = h->bias[l];
+  }
+  p.head_w = h->head_w;
+  p.head_b = h->head_b;
+  p.out_t = out_t;
+  p.out_hit = out_hit;
+  p.out_steps = out_steps;
+  p.queue = h->trc_queue;
+  p.status = h->status_dev;
+  p.timeout_ns = h->timeout_ns;
+  ProfScope ps(h, kProfGemm, st);
+  DDF_CK(ddf::launch_tc_trace(h->cfg.octaves, W, maps, p, h->trc_clusters, st));
+  return DDF_OK;
+}
+
 }  // namespace ddfi
 
 using namespace ddfi;
@@ -789,6 +837,9 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
   DeviceGuard g(h->cfg.device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int W = h->cfg.width, H = h->cfg.hidden_layers, cap = static_cast<int>(n);
+  if (h->trc_clusters < 0) h->trc_clusters = ddf::tc_trace_clusters(h->cfg.octaves, W, H);
+  if (h->trc_clusters > 0 && h->tile_auto && n <= kTraceRays)
+    return trace_in_one(h, rays, cap, max_steps, eps, t_max, out_t, out_hit, out_steps, st);
   if ((s = ensure_workspace(h, cap)) != DDF_OK) return s;
   if ((s = ensure_trace_buffers(h, cap)) != DDF_OK) return s;
   if ((s = ensure_plain_maps(h)) != DDF_OK) return s;

@@ -152,6 +152,9 @@ struct ddf_s {
   std::vector<CUtensorMap> tmBpair, tmWTpair;
 
   // sphere tracing (SDF fields)
+  int trc_clusters = -1;                  // of the one-kernel trace; 0: not for this field, -1: not asked
+  std::vector<CUtensorMap> tmTrace;
+  int* trc_queue = nullptr;
   int* trc_idx[2] = {nullptr, nullptr};   // active-ray lists
   int* trc_count = nullptr;               // [2] active counts
   int* trc_steps = nullptr;               // per-ray evaluations
@@ -207,6 +210,9 @@ constexpr int64_t kPairRows = 10240;
 inline int64_t small_rows(int width, int num_sms) {
   return 128 * (static_cast<int64_t>(2) * num_sms / (width / 64));
 }
+
+// Rays up to which a trace runs in one persistent kernel (TRACE_RULE).
+constexpr int64_t kTraceRays = int64_t{1} << 30;
 
 constexpr int kProfClasses = 4;
 enum ProfClass { kProfEncode = 0, kProfGemm = 1, kProfHead = 2, kProfFirst = 3 };

@@ -88,6 +88,31 @@ cudaError_t launch_trace_update(const float2* part, int nparts, int cap, const i
                                 const int* idx_in, const float* head_b, float eps, float t_max,
                                 int max_steps, float* t, int* steps, uint8_t* hit, int* idx_out,
                                 int* count_out, cudaStream_t s);
+// A whole trace in one persistent kernel (tc_trace.cu): SDF fields of width 128
+// .. 512 (a multiple of 128), 1 .. kTraceLayers layers. maps: every layer's bf16
+// weights with boxes of 64 K x 128 rows; queue: one device int of scratch.
+// Results are those of the step-by-step kernels, bit for bit.
+constexpr int kTraceLayers = 16;
+struct TraceMaps {
+  CUtensorMap m[kTraceLayers];
+};
+struct TraceParams {
+  RaySoA rays;
+  int n, L, H, max_steps;
+  float eps, t_max;
+  const float* bias[kTraceLayers];
+  const float* head_w;  // [W]
+  const float* head_b;  // [1]
+  float* out_t;
+  uint8_t* out_hit;
+  int* out_steps;  // nullable
+  int* queue;
+  uint32_t* status;
+  uint64_t timeout_ns;
+};
+int tc_trace_clusters(int L, int W, int H);
+cudaError_t launch_tc_trace(int L, int W, const TraceMaps& maps, const TraceParams& p, int clusters,
+                            cudaStream_t st);
 // Closed-form signed distance to a union of spheres and boxes at n points.
 cudaError_t launch_union_sdf(const float* spheres, int ns, const float* boxes, int nb,
                              const float* px, const float* py, const float* pz, int64_t n,

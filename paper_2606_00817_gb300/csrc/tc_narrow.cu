@@ -108,12 +108,17 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
   // The producer thread: barriers, then weight chunks for as long as the ring
   // has room, before the rest of the CTA is even set up.
   int64_t loaded = 0;  // chunks issued
-  int load_layer = 0, load_kb = 0;
+  int load_slot = 0, load_layer = 0, load_kb = 0;  // of the next one
+  uint32_t load_ph = 0;
   auto load_chunk = [&]() {
-    const int s = static_cast<int>(loaded % sh.slots);
-    mbar_arrive_expect_tx(full_bar(s), kChunk);
-    tma_load_2d(smem_u32(ring + s * kChunk), p.maps + load_layer, load_kb * 64, 0, full_bar(s));
+    mbar_arrive_expect_tx(full_bar(load_slot), kChunk);
+    tma_load_2d(smem_u32(ring + load_slot * kChunk), p.maps + load_layer, load_kb * 64, 0,
+                full_bar(load_slot));
     ++loaded;
+    if (++load_slot == sh.slots) {
+      load_slot = 0;
+      load_ph ^= 1u;
+    }
     if (++load_kb == (load_layer == 0 ? sh.kb1 : kbh)) {
       load_kb = 0;
       load_layer = load_layer + 1 == p.H ? 0 : load_layer + 1;
@@ -205,19 +210,21 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
     if (lane == 0) {
       bool ok = true;
       while (loaded < total) {
-        const int s = static_cast<int>(loaded % sh.slots);
-        const uint32_t ph = static_cast<uint32_t>((loaded / sh.slots) & 1);
-        if (!mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, p.timeout_ns)) {
+        if (!mbar_wait_bounded(empty_bar(load_slot), load_ph ^ 1u, abort_flag, p.timeout_ns)) {
           ok = false;
           break;
         }
         load_chunk();
       }
       if (!ok) raise_abort();
-      // no exit with a copy in flight
-      for (int64_t j = loaded > sh.slots ? loaded - sh.slots : 0; j < loaded; ++j)
-        mbar_wait_bounded(full_bar(static_cast<int>(j % sh.slots)),
-                          static_cast<uint32_t>((j / sh.slots) & 1), nullptr, kNwDrainNs);
+      // no exit with a copy in flight: back over the last chunks
+      for (int64_t j = loaded < sh.slots ? loaded : sh.slots; j > 0; --j) {
+        if (--load_slot < 0) {
+          load_slot = sh.slots - 1;
+          load_ph ^= 1u;
+        }
+        mbar_wait_bounded(full_bar(load_slot), load_ph, nullptr, kNwDrainNs);
+      }
     }
   } else {
     const uint32_t a0 = smem_u32(sA);
@@ -241,7 +248,8 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
           : "memory");
       return all != 0;
     };
-    int64_t it = 0;       // streamed: chunks consumed
+    int slot = 0;         // streamed: the next chunk's, and its phase (64-bit counters
+    uint32_t sph = 0;     // and their divisions cost 400 cycles a chunk)
     uint32_t dphase = 0;  // layers finished, mod 2
     bool ok = true;
     for (int64_t tile = tile0; tile < tiles && ok;
@@ -255,9 +263,9 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
           tc_fence_after();
           const int kbs = l == 0 ? sh.kb1 : kbh;
           const int first = l == 0 ? 0 : sh.kb1 + (l - 1) * kbh;
-          for (int kb = 0; kb < kbs && ok; ++kb, ++it) {
-            const int s = sh.resident ? first + kb : static_cast<int>(it % sh.slots);
-            const uint32_t ph = sh.resident ? 0u : static_cast<uint32_t>((it / sh.slots) & 1);
+          for (int kb = 0; kb < kbs && ok; ++kb) {
+            const int s = sh.resident ? first + kb : slot;
+            const uint32_t ph = sh.resident ? 0u : sph;
             if (!mbar_wait_bounded(full_bar(s), ph, abort_flag, p.timeout_ns)) {
               ok = false;
               break;
@@ -268,7 +276,13 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
             for (int j = 0; j < 4; ++j)
               tc_mma_f16(d_tmem, sw128_kmajor_desc(ab + 32u * j), sw128_kmajor_desc(bb + 32u * j),
                          idesc, (kb != 0 || j != 0) ? 1u : 0u);
-            if (!sh.resident) tc_commit(empty_bar(s));
+            if (!sh.resident) {
+              tc_commit(empty_bar(s));
+              if (++slot == sh.slots) {
+                slot = 0;
+                sph ^= 1u;
+              }
+            }
           }
           tc_commit(done_bar(g));  // arrives once every MMA above has finished
           ok = mbar_wait_bounded(done_bar(g), dphase, nullptr, p.timeout_ns) && ok;
