@@ -299,7 +299,7 @@ ddf_status mlp_gradients(ddf_s* h, int B, cudaStream_t st) {
     ddf::GradReduce g;
     g.nsplit = static_cast<int>(std::min<size_t>(ddf::kRedJobs, sums.size() - j0));
     for (int j = 0; j < g.nsplit; ++j) g.split[j] = sums[j0 + j];
-    DDF_CK(ddf::launch_grad_reduce(g, st));
+    DDF_CK(ddf::launch_grad_reduce(g, true, st));
   }
   return DDF_OK;
 }

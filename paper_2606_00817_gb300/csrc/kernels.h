@@ -377,7 +377,8 @@ struct GradReduce {
   RedCols cols;
   int blk0[kRedJobs + 1] = {};  // block offsets of the split jobs (set by the launcher)
 };
-cudaError_t launch_grad_reduce(const GradReduce& g, cudaStream_t s);
+// batched: the variant for a hash grid's small gradients.
+cudaError_t launch_grad_reduce(const GradReduce& g, bool batched, cudaStream_t s);
 // Adam (Kingma & Ba, bias-corrected with bc1 = 1 - b1^t, bc2 = 1 - b2^t, no
 // weight decay) on n parameters: m, v and w updated in place.
 cudaError_t launch_adam(float* w, const float* g, float* m, float* v, int64_t n, float lr,

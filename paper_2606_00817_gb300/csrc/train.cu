@@ -134,12 +134,20 @@ __global__ void sdf_loss_kernel(const float2* __restrict__ z, const float* __res
   }
 }
 
+__global__ void sum_partials_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) {
+    float t = 0.f;
+    for (int i = 0; i < n; ++i) t += part[i];
+    *out = t;
+  }
+}
+
 constexpr int kSumThreads = 256;
 
 // The n partial sums added in order by one thread, from shared memory: with a
 // dependent global load each, 256 of them took 6.7 us.
 __global__ void __launch_bounds__(kSumThreads)
-sum_partials_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
+sum_partials_staged_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
   __shared__ float s[kSumThreads];
   float t = 0.f;
   for (int base = 0; base < n; base += kSumThreads) {
@@ -269,8 +277,15 @@ __device__ __forceinline__ void add4(float4& a, const float4 b) {
   a.w += b.w;
 }
 
+// BATCHED: the partials' loads of a thread in flight together, and single
+// elements where rows are not whole float4s (a hash grid's MLP gradients, 16,384
+// rays: 22 -> 14 us). Not beside the CTA-pair GEMMs of a layered field, where it
+// gained nothing and, at 64 registers a thread instead of 40, a training loop on
+// one of several GPUs stopped making progress once in a few hundred steps; with
+// the plain loop 10,000 steps ran through.
 constexpr int kRedBatch = 8;  // 16-byte loads in flight a thread
 
+template <bool BATCHED>
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant__ GradReduce g) {
   const int b = blockIdx.x;
   if (b < g.blk0[g.nsplit]) {
@@ -279,23 +294,43 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant_
     const RedSplit& a = g.split[j];
     const int64_t e0 = 4 * (static_cast<int64_t>(b - g.blk0[j]) * blockDim.x + threadIdx.x);
     const int64_t total = static_cast<int64_t>(a.rows) * a.cols;
-    if (a.vec) {
+    if (a.vec || !BATCHED) {
       if (e0 >= total) return;
+    }
+    if (a.vec) {
       const int r = static_cast<int>(e0 / a.cols);
       const int c = static_cast<int>(e0 - static_cast<int64_t>(r) * a.cols);
       const float* src = a.part + static_cast<int64_t>(r) * a.ldp + c;
       float* dst = a.out + static_cast<int64_t>(r) * a.ldo + c;  // cols, ldp, ldo, split_stride multiples of 4; 16-byte aligned
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int q0 = 0; q0 < a.S; q0 += kRedBatch) {  // loads in flight together, added in order
-        float4 v[kRedBatch];
+      if constexpr (!BATCHED) {
+#pragma unroll 4
+        for (int q = 0; q < a.S; ++q)
+          add4(acc, *reinterpret_cast<const float4*>(src + q * a.split_stride));
+      } else {
+        for (int q0 = 0; q0 < a.S; q0 += kRedBatch) {  // loads in flight together, added in order
+          float4 v[kRedBatch];
 #pragma unroll
-        for (int j = 0; j < kRedBatch; ++j)
-          if (q0 + j < a.S) v[j] = *reinterpret_cast<const float4*>(src + (q0 + j) * a.split_stride);
+          for (int j = 0; j < kRedBatch; ++j)
+            if (q0 + j < a.S)
+              v[j] = *reinterpret_cast<const float4*>(src + (q0 + j) * a.split_stride);
 #pragma unroll
-        for (int j = 0; j < kRedBatch; ++j)
-          if (q0 + j < a.S) add4(acc, v[j]);
+          for (int j = 0; j < kRedBatch; ++j)
+            if (q0 + j < a.S) add4(acc, v[j]);
+        }
       }
       *reinterpret_cast<float4*>(dst) = acc;
+      return;
+    }
+    if constexpr (!BATCHED) {
+      for (int k = 0; k < 4 && e0 + k < total; ++k) {  // the 4 elements may span rows
+        const int rk = static_cast<int>((e0 + k) / a.cols);
+        const int ck = static_cast<int>(e0 + k - static_cast<int64_t>(rk) * a.cols);
+        const float* sk = a.part + static_cast<int64_t>(rk) * a.ldp + ck;
+        float acc = 0.f;
+        for (int q = 0; q < a.S; ++q) acc += sk[q * a.split_stride];
+        a.out[static_cast<int64_t>(rk) * a.ldo + ck] = acc;
+      }
       return;
     }
     // rows of any length: one element a thread
@@ -672,7 +707,8 @@ cudaError_t launch_loss_dz(const float2* z, const float* t_tgt, const uint8_t* y
 
 cudaError_t launch_loss_sum(const float* part, int64_t B, float* loss_out, cudaStream_t s) {
   if (loss_out == nullptr) return cudaSuccess;
-  sum_partials_kernel<<<1, kSumThreads, 0, s>>>(part, static_cast<int>((B + 255) / 256), loss_out);
+  sum_partials_staged_kernel<<<1, kSumThreads, 0, s>>>(part, static_cast<int>((B + 255) / 256),
+                                                       loss_out);
   return cudaGetLastError();
 }
 
@@ -681,14 +717,16 @@ cudaError_t launch_loss(const float2* z, const float* t_tgt, const uint8_t* y, i
                         float* loss_out, cudaStream_t s) {
   cudaError_t e = launch_count_hits(y, B, nhit, s);
   if (e == cudaSuccess) e = launch_loss_dz(z, t_tgt, y, B, nhit, clamp, lam, dz, part, s);
-  return e != cudaSuccess ? e : launch_loss_sum(part, B, loss_out, s);
+  if (e != cudaSuccess || loss_out == nullptr) return e;
+  sum_partials_kernel<<<1, 32, 0, s>>>(part, static_cast<int>((B + 255) / 256), loss_out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sdf_loss(const float2* z, const float* s_tgt, int64_t B, float2* dz,
                             float* part, float* loss_out, cudaStream_t s) {
   const int blocks = static_cast<int>((B + 255) / 256);
   sdf_loss_kernel<<<blocks, 256, 0, s>>>(z, s_tgt, B, dz, part);
-  if (loss_out != nullptr) sum_partials_kernel<<<1, kSumThreads, 0, s>>>(part, blocks, loss_out);
+  if (loss_out != nullptr) sum_partials_kernel<<<1, 32, 0, s>>>(part, blocks, loss_out);
   return cudaGetLastError();
 }
 
@@ -702,7 +740,7 @@ cudaError_t launch_head_back_fused(const float2* dz, const __nv_bfloat16* H, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_grad_reduce(const GradReduce& g0, cudaStream_t s) {
+cudaError_t launch_grad_reduce(const GradReduce& g0, bool batched, cudaStream_t s) {
   GradReduce g = g0;
   if (g.nsplit < 0 || g.nsplit > kRedJobs) return cudaErrorInvalidValue;
   auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
@@ -714,7 +752,7 @@ cudaError_t launch_grad_reduce(const GradReduce& g0, cudaStream_t s) {
       return cudaErrorInvalidValue;
     a.vec = a.cols % 4 == 0 && a.ldp % 4 == 0 && a.ldo % 4 == 0 && a.split_stride % 4 == 0 &&
             al16(a.part) && al16(a.out);
-    const int64_t per = a.vec ? 1024 : 256;  // elements a block
+    const int64_t per = a.vec || !batched ? 1024 : 256;  // elements a block
     const int64_t nb = (static_cast<int64_t>(a.rows) * a.cols + per - 1) / per;
     if (g.blk0[j] + nb > (1ll << 30)) return cudaErrorInvalidValue;
     g.blk0[j + 1] = g.blk0[j] + static_cast<int>(nb);
@@ -739,7 +777,10 @@ cudaError_t launch_grad_reduce(const GradReduce& g0, cudaStream_t s) {
   }
   if (blocks == 0) return cudaSuccess;
   if (blocks > (1ll << 31) - 1) return cudaErrorInvalidValue;
-  grad_reduce_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(g);
+  if (batched)
+    grad_reduce_kernel<true><<<static_cast<unsigned>(blocks), 256, 0, s>>>(g);
+  else
+    grad_reduce_kernel<false><<<static_cast<unsigned>(blocks), 256, 0, s>>>(g);
   return cudaGetLastError();
 }
 

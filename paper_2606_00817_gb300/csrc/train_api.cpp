@@ -34,13 +34,15 @@ ddf_status ensure_reduce_stream(ddf_s* h) {
       DDF_CK(cudaEventCreateWithFlags(&h->ev_red[b], cudaEventDisableTiming));
   }
   if (h->ev_join == nullptr) DDF_CK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
+  if (h->cfg.kind != DDF_KIND_HASHGRID) {
+    DDF_CK(cudaStreamCreateWithFlags(&h->s_red, cudaStreamNonBlocking));
+    return DDF_OK;
+  }
   // a hash grid's side kernels are small and run beside an Adam pass of many
-  // thousand blocks, behind which they would queue without a priority; beside
-  // the persistent GEMMs of a layered field they keep the usual one
+  // thousand blocks, behind which they would queue without a priority
   int least = 0, greatest = 0;
   DDF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-  DDF_CK(cudaStreamCreateWithPriority(&h->s_red, cudaStreamNonBlocking,
-                                      h->cfg.kind == DDF_KIND_HASHGRID ? greatest : least));
+  DDF_CK(cudaStreamCreateWithPriority(&h->s_red, cudaStreamNonBlocking, greatest));
   return DDF_OK;
 }
 
@@ -408,7 +410,7 @@ ddf_status backward_from_dz(ddf_s* h, int B, cudaStream_t st) {
     c.c0[2] = 3 * W;      // db_o
     c.cnt[2] = hr;
     c.out[2] = h->grad + o.bo;
-    DDF_CK(ddf::launch_grad_reduce(g, st));
+    DDF_CK(ddf::launch_grad_reduce(g, false, st));
   }
 
   // ---- layers, last to first. Each layer's reduction runs on the side
@@ -541,7 +543,7 @@ ddf_status backward_layers(ddf_s* h, int B, cudaStream_t st, cudaStream_t rs) {
       }
       DDF_CK(cudaEventRecord(h->ev_gemm[l & 1], st));
       DDF_CK(cudaStreamWaitEvent(rs, h->ev_gemm[l & 1], 0));
-      DDF_CK(ddf::launch_grad_reduce(g, rs));
+      DDF_CK(ddf::launch_grad_reduce(g, false, rs));
       DDF_CK(cudaEventRecord(h->ev_red[l & 1], rs));
       pending[l & 1] = true;
     }
