@@ -122,6 +122,7 @@ void release_weight_buffers(ddf_s* h) {
   h->tmBig.clear();
   h->tmSmall.clear();
   h->tmTrace.clear();
+  h->tmStep.clear();
   h->wcal.clear();
   h->wp.clear();
   h->wq.clear();
@@ -726,6 +727,20 @@ ddf_status ensure_plain_maps(ddf_s* h) {
   return DDF_OK;
 }
 
+// Weight maps of the narrow tiles of a tracing step.
+ddf_status ensure_step_maps(ddf_s* h) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  if (static_cast<int>(h->tmStep.size()) == H) return DDF_OK;
+  std::vector<CUtensorMap> maps(H);
+  for (int l = 0; l < H; ++l) {
+    const int kp = l == 0 ? h->kp16 : W;
+    if (!make_tmap(&maps[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2, 64))
+      return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
+  }
+  h->tmStep = maps;
+  return DDF_OK;
+}
+
 ddf_status ensure_trace_buffers(ddf_s* h, int64_t rows) {
   if (rows <= h->trc_rows) return DDF_OK;
   dev_free(h, h->trc_idx[0]);
@@ -741,6 +756,14 @@ ddf_status ensure_trace_buffers(ddf_s* h, int64_t rows) {
   }
   if ((s = dev_alloc(h, &p, rows * sizeof(int))) != DDF_OK) return s;
   h->trc_steps = static_cast<int*>(p);
+  // FP32 activations of the last layer in steps with few rays (128 wide tiles at worst)
+  dev_free(h, h->trc_x);
+  h->trc_x = nullptr;
+  const int64_t xr = std::min<int64_t>(
+      round_up(rows, 128), std::max(ddf::step_small_rows(h->cfg.width, 128, h->num_sms),
+                                    ddf::step_small_rows(h->cfg.width, h->bn, h->num_sms)));
+  if ((s = dev_alloc(h, &p, xr * h->cfg.width * sizeof(float))) != DDF_OK) return s;
+  h->trc_x = static_cast<float*>(p);
   if (h->trc_count == nullptr) {
     if ((s = dev_alloc(h, &p, 2 * sizeof(int))) != DDF_OK) return s;
     h->trc_count = static_cast<int*>(p);
@@ -838,36 +861,37 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int W = h->cfg.width, H = h->cfg.hidden_layers, cap = static_cast<int>(n);
   if (h->trc_clusters < 0) h->trc_clusters = ddf::tc_trace_clusters(h->cfg.octaves, W, H);
-  if (h->trc_clusters > 0 && h->tile_auto && n <= kTraceRays)
+  if (h->trc_clusters > 0 && h->tile_auto && n <= trace_rays(W, h->trc_clusters))
     return trace_in_one(h, rays, cap, max_steps, eps, t_max, out_t, out_hit, out_steps, st);
   if ((s = ensure_workspace(h, cap)) != DDF_OK) return s;
   if ((s = ensure_trace_buffers(h, cap)) != DDF_OK) return s;
   if ((s = ensure_plain_maps(h)) != DDF_OK) return s;
+  if ((s = ensure_step_maps(h)) != DDF_OK) return s;
+  std::vector<CUtensorMap> tmA(H);
+  for (int l = 0; l < H; ++l) {
+    const int K = l == 0 ? h->kp16 : W;
+    if (!make_tmap(&tmA[l], l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1], false, K, cap,
+                   static_cast<uint64_t>(K) * 2, 128))
+      return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
+  }
   int* steps = out_steps != nullptr ? out_steps : h->trc_steps;
   ddf::RaySoA r;
   for (int c = 0; c < 6; ++c) r.p[c] = rays[c];
-  const ddf::TcTile tile{h->bn, 4};
-  const int64_t max_tiles = ((cap + 127) / 128) * static_cast<int64_t>(W / tile.bn);
-  const int grid = static_cast<int>(std::min<int64_t>(max_tiles, h->num_sms));
+  const int bn = h->bn;
   DDF_CK(ddf::launch_trace_init(cap, h->trc_idx[0], h->trc_count, out_t, steps, out_hit, st));
   for (int it = 0; it < max_steps; ++it) {
     int* cin = h->trc_count + (it & 1);
     int* cout = h->trc_count + ((it + 1) & 1);
     const int* iin = h->trc_idx[it & 1];
     int* iout = h->trc_idx[(it + 1) & 1];
-    DDF_CK(cudaMemsetAsync(cout, 0, sizeof(int), st));
     {
       ProfScope ps(h, kProfEncode, st);
-      DDF_CK(ddf::launch_trace_encode(r, out_t, iin, cin, cap, h->cfg.octaves, h->kp16,
-                                      static_cast<__nv_bfloat16*>(h->ws_enc), st));
+      DDF_CK(ddf::launch_step_encode(r, out_t, iin, cin, cout, cap, h->cfg.octaves, h->kp16,
+                                     static_cast<__nv_bfloat16*>(h->ws_enc), h->num_sms, it == 0, st));
     }
     for (int l = 0; l < H; ++l) {
       const bool last = l == H - 1;
-      const void* a_base = l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1];
       const int K = l == 0 ? h->kp16 : W;
-      CUtensorMap tmA;
-      if (!make_tmap(&tmA, a_base, false, K, cap, static_cast<uint64_t>(K) * 2, 128))
-        return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
       ddf::TcGemmParams p{};
       p.M = cap;
       p.m_dev = cin;
@@ -879,15 +903,35 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
       p.ldo = W;
       p.head_w = h->head_w;
       p.head_part = h->ws_part;
+      p.out_f32 = last ? h->trc_x : nullptr;
       p.mode = last ? 1 : 0;
       p.status = h->status_dev;
       p.timeout_ns = h->timeout_ns;
       ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
-      DDF_CK(ddf::launch_tc_gemm(tile, false, false, tmA, h->tmBtr[l], p, grid, st));
+      DDF_CK(ddf::launch_step_layer(tmA[l], h->tmBtr[l], h->tmStep[l], p, bn, h->num_sms,
+                                    it == 0 && (l == 0 || last), st));
     }
     ProfScope ps(h, kProfHead, st);
-    DDF_CK(ddf::launch_trace_update(h->ws_part, W / tile.bn, cap, cin, iin, h->head_b, eps, t_max,
-                                    max_steps, out_t, steps, out_hit, iout, cout, st));
+    ddf::StepUpdate u{};
+    u.part = h->ws_part;
+    u.x = h->trc_x;
+    u.head_w = h->head_w;
+    u.head_b = h->head_b;
+    u.N = W;
+    u.bn = bn;
+    u.cap = cap;
+    u.sms = h->num_sms;
+    u.max_steps = max_steps;
+    u.eps = eps;
+    u.t_max = t_max;
+    u.count_in = cin;
+    u.idx_in = iin;
+    u.t = out_t;
+    u.steps = steps;
+    u.hit = out_hit;
+    u.idx_out = iout;
+    u.count_out = cout;
+    DDF_CK(ddf::launch_step_update(u, it == 0, st));
   }
   return DDF_OK;
 }
@@ -1532,6 +1576,7 @@ ddf_status ddf_set_tile(ddf_handle h, int32_t which, const ddf_tile* tile) {
   clear_graphs(h);  // weight maps and launch shapes change
   (which == 1 ? h->tile_first : h->tile) =
       ddf::TcTile{bn, ew, tile->cta_pair != 0, tile->staged != 0, tile->fused_encode != 0};
+  if (h->bn != h->tile.bn) h->tmBtr.clear();  // boxes of the old bn
   h->bn = h->tile.bn;
   h->tile_auto = false;
   if (h->loaded && h->cfg.precision != DDF_FP32) {

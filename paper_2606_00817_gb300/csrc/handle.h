@@ -153,7 +153,8 @@ struct ddf_s {
 
   // sphere tracing (SDF fields)
   int trc_clusters = -1;                  // of the one-kernel trace; 0: not for this field, -1: not asked
-  std::vector<CUtensorMap> tmTrace;
+  std::vector<CUtensorMap> tmTrace, tmStep;
+  float* trc_x = nullptr;
   int* trc_queue = nullptr;
   int* trc_idx[2] = {nullptr, nullptr};   // active-ray lists
   int* trc_count = nullptr;               // [2] active counts
@@ -211,8 +212,17 @@ inline int64_t small_rows(int width, int num_sms) {
   return 128 * (static_cast<int64_t>(2) * num_sms / (width / 64));
 }
 
-// Rays up to which a trace runs in one persistent kernel (TRACE_RULE).
-constexpr int64_t kTraceRays = int64_t{1} << 30;
+// Rays up to which a trace runs in one persistent kernel of `clusters` clusters
+// of 128 lanes (tc_trace.cu): as many as it has lanes, twice as many at widths
+// up to 256. A round of its lanes takes about 40 us at 512 x 6 and 15 us at 256 x
+// 4, a step of the step kernels with few rays 30 and 15 us, so for the first
+// rays it wins (512 x 6, 3,000 rays 2.34 and 2.93 ms; 256 x 4, 3,000 rays 1.07 and
+// 1.97 ms); with more rays than lanes it would lose on fields whose rays all
+// take many steps, even where it wins on others (256 x 4, 65,536 rays of 8 steps
+// 1.88 and 2.76 ms; 512 x 6 7.6 and 5.1 ms).
+inline int64_t trace_rays(int width, int clusters) {
+  return int64_t{128} * clusters * (width <= 256 ? 2 : 1);
+}
 
 constexpr int kProfClasses = 4;
 enum ProfClass { kProfEncode = 0, kProfGemm = 1, kProfHead = 2, kProfFirst = 3 };

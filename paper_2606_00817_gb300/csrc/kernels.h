@@ -73,21 +73,9 @@ struct TcGemmParams {
 // band sin(pi 2^k p_c), cos(pi 2^k p_c); zero padding to ld.
 cudaError_t launch_encode_points_bf16(const float* px, const float* py, const float* pz, int64_t M,
                                       int L, int ld, __nv_bfloat16* out, cudaStream_t s);
-// Same for the active rays of a trace: row j encodes o_i + t_i d_i with
-// i = idx[j], for j < *count (rows up to cap written, extra rows untouched).
-cudaError_t launch_trace_encode(RaySoA rays, const float* t, const int* idx, const int* count,
-                                int cap, int L, int ld, __nv_bfloat16* out, cudaStream_t s);
 // idx = 0..n-1, count = n, t = 0, steps = 0, hit = 0
 cudaError_t launch_trace_init(int n, int* idx, int* count, float* t, int* steps, uint8_t* hit,
                               cudaStream_t s);
-// One sphere-tracing step for the active rays: s = sum of nparts head
-// partials [nparts x cap] + head_b[0]; steps += 1; s < eps -> hit; else
-// t += s and the ray stays active (appended to idx_out / count_out) unless
-// t > t_max or it has used max_steps evaluations.
-cudaError_t launch_trace_update(const float2* part, int nparts, int cap, const int* count_in,
-                                const int* idx_in, const float* head_b, float eps, float t_max,
-                                int max_steps, float* t, int* steps, uint8_t* hit, int* idx_out,
-                                int* count_out, cudaStream_t s);
 // A whole trace in one persistent kernel (tc_trace.cu): SDF fields of width 128
 // .. 512 (a multiple of 128), 1 .. kTraceLayers layers. maps: every layer's bf16
 // weights with boxes of 64 K x 128 rows; queue: one device int of scratch.
@@ -113,6 +101,37 @@ struct TraceParams {
 int tc_trace_clusters(int L, int W, int H);
 cudaError_t launch_tc_trace(int L, int W, const TraceMaps& maps, const TraceParams& p, int clusters,
                             cudaStream_t st);
+// The kernels of one tracing step on a device-side count (tc_steps.cu), each
+// launched with programmatic dependence on the one before it; sms: the device's
+// SMs, the same for all. A step is launch_step_encode (which also clears
+// next_count), launch_step_layer for every layer, launch_step_update. The layer
+// takes 128 x bn tiles (tmB: boxes of bn rows) where the count fills the SMs, else
+// 128 x 64 tiles (tmB64: boxes of 64 rows); the last one (p.mode 1) then writes
+// FP32 activations to p.out_f32 [step_small_rows x N] instead of head partials.
+int64_t step_small_rows(int N, int bn, int sms);
+// first: the first step of a trace, which configures the kernels.
+cudaError_t launch_step_encode(const RaySoA& rays, const float* t, const int* idx, const int* count,
+                               int* next_count, int cap, int L, int ld, __nv_bfloat16* out, int sms,
+                               bool first, cudaStream_t s);
+cudaError_t launch_step_layer(const CUtensorMap& tmA, const CUtensorMap& tmB,
+                              const CUtensorMap& tmB64, const TcGemmParams& p, int bn, int sms,
+                              bool first, cudaStream_t s);
+struct StepUpdate {
+  const float2* part;  // [N / bn x cap]
+  const float* x;      // [rows x N]
+  const float* head_w;
+  const float* head_b;
+  int N, bn, cap, sms, max_steps;
+  float eps, t_max;
+  const int* count_in;
+  const int* idx_in;
+  float* t;
+  int* steps;
+  uint8_t* hit;
+  int* idx_out;
+  int* count_out;
+};
+cudaError_t launch_step_update(const StepUpdate& u, bool first, cudaStream_t s);
 // Closed-form signed distance to a union of spheres and boxes at n points.
 cudaError_t launch_union_sdf(const float* spheres, int ns, const float* boxes, int nb,
                              const float* px, const float* py, const float* pz, int64_t n,

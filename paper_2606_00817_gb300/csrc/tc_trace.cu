@@ -18,7 +18,9 @@
 // the chain of a step: per layer the MMAs (2,048 cycles at W = 512), a cluster
 // handshake, the epilogue and the copies. (Storing the outputs to the peers from
 // the registers, 16 bytes a thread, took 9,500 cycles a layer.)
-// 65,536 rays through 51 -> 512 x 6, 8.4 steps a ray, 77 at most: TRACE_US.
+// Up to 128 steps, 8.4 a ray: 300 rays through 39 -> 256 x 4 3.97 -> 0.59 ms,
+// 3,000 rays 4.59 -> 1.07; through 51 -> 512 x 6 6.46 -> 2.34 and 6.58 -> 2.34. Larger
+// batches take the step kernels (tc_steps.cu).
 //
 // The arithmetic is that of the layer kernels in their order, so t, hit and
 // steps are the same bits: K ascending, ReLU(acc + b) rounded to bf16, the head's

@@ -106,3 +106,27 @@ def test_random_field_and_weights_loaded_again(cuda_lib):
         b.load(blob)
         for u, v in zip(_trace(ddf, a, rays, 5000, 40), _trace(ddf, b, rays, 5000, 40)):
             assert torch.equal(u, v)
+
+
+@pytest.mark.parametrize("net", [(4, 640, 2), (10, 1280, 3), (4, 2048, 2)])
+@pytest.mark.parametrize("n", [1, 129, 2304, 2305, 3840, 3841, 9000])
+def test_step_kernels_where_their_tiles_change(cuda_lib, net, n):
+    """Wide fields: a trace of one step moves each ray by the field's value at
+    its origin, as ddf_sdf_eval has it, or reports a hit (an output bias of 0: a
+    trace adds it before the head's blocks, ddf_sdf_eval after them); with more
+    steps a ray's trace does not depend on the batch, so on the tiles its steps
+    take."""
+    import torch
+    rays = _rays(torch, n, seed=n)
+    ddf, a, _ = _pair(net, _sphere_blob(net, seed=n, radius=0.0))
+    s = torch.empty(n, device="cuda")
+    ddf.ddf_sdf_eval(a.h, rays[:3], n, s, torch.cuda.current_stream())
+    t, hit, steps = _trace(ddf, a, rays, n, 1, 0.5, 1e6)
+    assert torch.equal(hit.bool(), s < 0.5) and bool((steps == 1).all())
+    assert torch.equal(t, torch.where(s < 0.5, torch.zeros_like(s), s))
+    ddf, a, _ = _pair(net, _sphere_blob(net, seed=n))
+    x = _trace(ddf, a, rays, n)
+    k = max(1, n // 3)
+    y = _trace(ddf, a, [r[n - k:].clone() for r in rays], k)
+    for u, v in zip(x, y):
+        assert torch.equal(u[n - k:], v)
