@@ -385,6 +385,51 @@ ddf_status forward_small(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cu
   return DDF_OK;
 }
 
+// A few thousand rays through a wide bf16 or e4m3 field (tc_steps.cu).
+ddf_status forward_mid(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
+  const int W = h->cfg.width, H = h->cfg.hidden_layers;
+  const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
+  // the buffer the last layer would write holds its split tiles
+  float* const x = static_cast<float*>(h->ws_act[(H - 1) & 1]);
+  const int64_t x_bytes = static_cast<int64_t>(m) * W * (fp8 ? 1 : 2);
+  const ddf::StepTiles mid{W / h->bn, h->bn == 256 ? 8 : 7, h->num_sms, h->num_sms};
+  ddf::StepTiles end = mid;
+  end.x_tiles = static_cast<int>(x_bytes / (128 * 4 * h->bn));
+  {
+    ProfScope ps(h, kProfEncode, st);
+    DDF_CK(ddf::launch_small_encode(rays, m, h->cfg.octaves, h->kp16,
+                                    static_cast<__nv_bfloat16*>(h->ws_enc), st));
+  }
+  for (int l = 0; l < H; ++l) {
+    const bool in_fp8 = fp8 && l > 0, last = l == H - 1, out_fp8 = fp8 && !last;
+    ddf::TcGemmParams p{};
+    p.M = m;
+    p.N = W;
+    p.K = l == 0 ? h->kp16 : W;
+    p.bias = h->bias[l];
+    p.col_scale = in_fp8 ? h->colscale[l] : nullptr;
+    p.out_scale = out_fp8 ? 1.0f / h->act_scales[l] : 1.0f;
+    p.out = h->ws_act[l & 1];
+    p.ldo = W;
+    p.head_w = h->head_w;
+    p.head_part = h->ws_part;
+    p.out_f32 = last ? x : nullptr;
+    p.mode = last ? 1 : 0;
+    p.status = h->status_dev;
+    p.timeout_ns = h->timeout_ns;
+    CUtensorMap tmA;
+    if (!make_tmap(&tmA, l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1], in_fp8, p.K, m,
+                   static_cast<uint64_t>(p.K) * (in_fp8 ? 1 : 2), 128))
+      return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
+    ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
+    DDF_CK(ddf::launch_step_layer(in_fp8, out_fp8, tmA, h->tmB[l], h->tmSmall[l], p,
+                                  last ? end : mid, true, st));
+  }
+  ProfScope ps(h, kProfHead, st);
+  DDF_CK(ddf::launch_step_heads(h->ws_part, x, m, end, h->head_w, h->head_b, out, st));
+  return DDF_OK;
+}
+
 ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaStream_t st) {
   const int W = h->cfg.width;
   const int H = h->cfg.hidden_layers;
@@ -406,6 +451,8 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
   }
   if (h->tile_auto && !h->tmSmall.empty() && m <= small_rows(W, h->num_sms) && m <= h->ws_x_rows)
     return forward_small(h, rays, m, out, st);
+  if (h->tile_auto && !h->tmSmall.empty() && (h->tmBig.empty() || m < mid_rows(W, h->num_sms, fp8)))
+    return forward_mid(h, rays, m, out, st);
   // the tiles in force: those set, or by the batch where none were (kPairRows)
   const bool big = h->tile_auto && !h->tmBig.empty() && m >= kPairRows;
   ddf::TcTile tile_h = h->tile, tile_1 = h->tile_first;
@@ -756,13 +803,12 @@ ddf_status ensure_trace_buffers(ddf_s* h, int64_t rows) {
   }
   if ((s = dev_alloc(h, &p, rows * sizeof(int))) != DDF_OK) return s;
   h->trc_steps = static_cast<int*>(p);
-  // FP32 activations of the last layer in steps with few rays (128 wide tiles at worst)
+  // FP32 activations of the last layer's split tiles: fewer tiles than SMs
   dev_free(h, h->trc_x);
   h->trc_x = nullptr;
-  const int64_t xr = std::min<int64_t>(
-      round_up(rows, 128), std::max(ddf::step_small_rows(h->cfg.width, 128, h->num_sms),
-                                    ddf::step_small_rows(h->cfg.width, h->bn, h->num_sms)));
-  if ((s = dev_alloc(h, &p, xr * h->cfg.width * sizeof(float))) != DDF_OK) return s;
+  const int64_t xe = std::min<int64_t>(round_up(rows, 128) * h->cfg.width,
+                                       int64_t{128} * 256 * h->num_sms);
+  if ((s = dev_alloc(h, &p, xe * sizeof(float))) != DDF_OK) return s;
   h->trc_x = static_cast<float*>(p);
   if (h->trc_count == nullptr) {
     if ((s = dev_alloc(h, &p, 2 * sizeof(int))) != DDF_OK) return s;
@@ -877,7 +923,7 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
   int* steps = out_steps != nullptr ? out_steps : h->trc_steps;
   ddf::RaySoA r;
   for (int c = 0; c < 6; ++c) r.p[c] = rays[c];
-  const int bn = h->bn;
+  const ddf::StepTiles tiles{W / h->bn, h->bn == 256 ? 8 : 7, h->num_sms, h->num_sms};
   DDF_CK(ddf::launch_trace_init(cap, h->trc_idx[0], h->trc_count, out_t, steps, out_hit, st));
   for (int it = 0; it < max_steps; ++it) {
     int* cin = h->trc_count + (it & 1);
@@ -908,7 +954,7 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
       p.status = h->status_dev;
       p.timeout_ns = h->timeout_ns;
       ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
-      DDF_CK(ddf::launch_step_layer(tmA[l], h->tmBtr[l], h->tmStep[l], p, bn, h->num_sms,
+      DDF_CK(ddf::launch_step_layer(false, false, tmA[l], h->tmBtr[l], h->tmStep[l], p, tiles,
                                     it == 0 && (l == 0 || last), st));
     }
     ProfScope ps(h, kProfHead, st);
@@ -917,10 +963,8 @@ ddf_status ddf_sphere_trace(ddf_handle h, const float* const rays[6], int64_t n,
     u.x = h->trc_x;
     u.head_w = h->head_w;
     u.head_b = h->head_b;
-    u.N = W;
-    u.bn = bn;
+    u.tiles = tiles;
     u.cap = cap;
-    u.sms = h->num_sms;
     u.max_steps = max_steps;
     u.eps = eps;
     u.t_max = t_max;

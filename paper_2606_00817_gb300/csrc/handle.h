@@ -197,19 +197,28 @@ struct DeviceGuard {
 
 // Rows from which a field whose tiles nobody set takes the staged CTA-pair tile
 // for its hidden layers and the fused layer 1 (the same bits as the default
-// tiles): at 1280 x 8, default against these tiles, bf16 8,192 rows 248 and 242
-// us, 12,000 rows 313 and 289, 140,000 rows 2,217 and 1,965; e4m3 8,192 rows 177
-// and 173, 16,384 rows 230 and 230, 140,000 rows 1,227 and 1,123; at 512 x 6,
-// 8,192 rows 77 and 84, 12,000 rows 100 and 95. Below, a 256 x 256 tile leaves
-// too many SMs idle.
+// tiles), where the tiles of mid_rows do not exist (SDF values): at 512 x 6 and
+// 1280 x 8 the pair tile draws level with the default one at 8,192 to 12,000 rows;
+// below, a 256 x 256 tile leaves too many SMs idle.
 constexpr int64_t kPairRows = 10240;
 
+// Rows from which a ray field does: below, the kernels of tc_steps.cu, whose
+// layers start faster and whose last wave is cut smaller; from 6 waves of 128 x 256
+// tiles on (e4m3: 10, its waves being shorter) the pair tile's rate outweighs
+// that. tc_steps.cu and the pair tile: bf16 1280 x 8 20,000 rows (5.2 waves) 372
+// and 395 us, 28,000 (7.2) 496 and 488; 512 x 6 40,000 (4.1) 149 and 162, 65,536 (6.7)
+// 228 and 218; 2048 x 4 14,000 (5.8) 258 and 257; e4m3 1280 x 8 40,000 (10.3) 386 and
+// 421, 65,536 (16.8) 592 and 583; 512 x 6 100,000 (10.3) 249 and 247.
+inline int64_t mid_rows(int width, int num_sms, bool fp8) {
+  return int64_t{128} * (fp8 ? 10 : 6) * num_sms / ((width + 255) / 256);
+}
+
 // Rows up to which a field whose tiles nobody set runs its layers on 128 x 64
-// tiles (tc_small.cu): two waves of them. At 1280 x 8 bf16, these against the
-// default tiles: 800 rows 75 and 129 us, 1,000 rows 121 and 129, 1,920 rows 133
-// and 133; e4m3 1,920 rows 94 and 114; a third wave would lose.
+// tiles (tc_small.cu): one wave of them. At 1280 x 8 bf16, these against the
+// kernels of tc_steps.cu: 1 row 66 and 70 us, 890 rows 77 and 80, 1,000 rows (the
+// second wave) 123 and 85; e4m3 500 rows 52 and 58, 1,000 rows 84 and 64.
 inline int64_t small_rows(int width, int num_sms) {
-  return 128 * (static_cast<int64_t>(2) * num_sms / (width / 64));
+  return 128 * (static_cast<int64_t>(num_sms) / (width / 64));
 }
 
 // Rays up to which a trace runs in one persistent kernel of `clusters` clusters

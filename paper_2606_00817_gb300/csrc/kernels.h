@@ -101,27 +101,50 @@ struct TraceParams {
 int tc_trace_clusters(int L, int W, int H);
 cudaError_t launch_tc_trace(int L, int W, const TraceMaps& maps, const TraceParams& p, int clusters,
                             cudaStream_t st);
-// The kernels of one tracing step on a device-side count (tc_steps.cu), each
-// launched with programmatic dependence on the one before it; sms: the device's
-// SMs, the same for all. A step is launch_step_encode (which also clears
-// next_count), launch_step_layer for every layer, launch_step_update. The layer
-// takes 128 x bn tiles (tmB: boxes of bn rows) where the count fills the SMs, else
-// 128 x 64 tiles (tmB64: boxes of 64 rows); the last one (p.mode 1) then writes
-// FP32 activations to p.out_f32 [step_small_rows x N] instead of head partials.
-int64_t step_small_rows(int N, int bn, int sms);
+// How the kernels of tc_steps.cu cut a layer into tiles, from the number of rows
+// alone: whole waves of 128 x bn tiles (all of them narrower if there is not one),
+// and what is left over split into tiles of 64 columns where those are no more
+// than a wave. 1280 x 8 bf16, a whole call of 4,099 rays (165 tiles on 152 SMs): 13
+// tiles in 52 parts 132 us, whole 142; 5,100 rays (48 tiles left): whole 141, in 192
+// parts (two waves) 179; parts of 128 columns instead lost to whole tiles (154).
+struct StepTiles {
+  int num_n;    // tiles of a row block: the width / bn
+  int lg_bn;    // bn = 1 << lg_bn: 128 or 256
+  int sms;
+  int x_tiles;  // a last layer: room for the FP32 activations of that many split tiles
+};
+struct TilePlan {
+  int big, lg_split, tiles;  // whole tiles; each one after them in 1 << lg_split; all tiles
+};
+__host__ __device__ inline TilePlan tile_plan(int rows, const StepTiles& s) {
+  const int all = (rows + 127) / 128 * s.num_n;
+  const int big = all < s.sms ? 0 : all / s.sms * s.sms, rest = all - big;
+  const int lg = s.lg_bn - 6;
+  if (rest > s.x_tiles || rest << lg > s.sms) return TilePlan{all, 0, all};
+  return TilePlan{big, lg, big + (rest << lg)};
+}
+// The kernels of one tracing step on a device-side count, or of a query
+// (tc_steps.cu), each launched with programmatic dependence on the one before
+// it; sms: the device's SMs, the same for all. A step is launch_step_encode
+// (which also clears next_count), launch_step_layer for every layer (tmB: boxes of
+// bn rows, tmB64: of 64), launch_step_update. The last layer (p.mode 1) writes head
+// partials, and where a tile is split FP32 activations to p.out_f32 [x_tiles x 128
+// x bn]; p.m_dev may be null: p.M rows.
 // first: the first step of a trace, which configures the kernels.
 cudaError_t launch_step_encode(const RaySoA& rays, const float* t, const int* idx, const int* count,
                                int* next_count, int cap, int L, int ld, __nv_bfloat16* out, int sms,
                                bool first, cudaStream_t s);
-cudaError_t launch_step_layer(const CUtensorMap& tmA, const CUtensorMap& tmB,
-                              const CUtensorMap& tmB64, const TcGemmParams& p, int bn, int sms,
-                              bool first, cudaStream_t s);
+cudaError_t launch_step_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
+                              const CUtensorMap& tmB, const CUtensorMap& tmB64,
+                              const TcGemmParams& p, const StepTiles& st, bool first,
+                              cudaStream_t s);
 struct StepUpdate {
   const float2* part;  // [N / bn x cap]
-  const float* x;      // [rows x N]
+  const float* x;      // split tiles' activations
   const float* head_w;
   const float* head_b;
-  int N, bn, cap, sms, max_steps;
+  StepTiles tiles;
+  int cap, max_steps;
   float eps, t_max;
   const int* count_in;
   const int* idx_in;
@@ -265,6 +288,9 @@ cudaError_t launch_small_encode(const RaySoA& rays, int64_t M, int L, int ld, __
                                 cudaStream_t s);
 cudaError_t launch_small_heads(const float* X, int M, int W, int blk, const float* wo,
                                const float* bo, const HeadOut& o, cudaStream_t s);
+// The heads after launch_step_layer's last layer: out_f32 as X, the same tiles.
+cudaError_t launch_step_heads(const float2* part, const float* X, int M, const StepTiles& st, const float* wo, const float* bo,
+                              const HeadOut& o, cudaStream_t s);
 // From per-N-block partial dot products [nblk x M] (tensor-core path).
 cudaError_t launch_finish_heads(const float2* part, int nblk, int M, const float* bo, HeadOut o,
                                 cudaStream_t s);

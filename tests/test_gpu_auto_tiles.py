@@ -78,3 +78,37 @@ def test_noalloc_follows_the_same_rule(cuda_lib):
         ddf.ddf_query_rays_noalloc(a.h, rays, n, t, v, torch.cuda.current_stream())
         rt, rv = b.query(rays)
         assert torch.equal(t, rt) and torch.equal(v, rv), n
+
+
+@pytest.mark.parametrize("net,precision", [((10, 1280, 3), "bf16"), ((10, 1280, 3), "fp8"),
+                                           ((8, 512, 2), "bf16"), ((10, 384, 3), "fp8")])
+@pytest.mark.parametrize("n", [2001, 3963, 4099, 4864, 4865, 5760, 5761, 7801, 9729])
+def test_layers_cut_into_whole_and_split_tiles(cuda_lib, net, precision, n):
+    """Between the small batches and the pair tiles: whole waves of wide tiles
+    and what is left of them split in two or four, with and without room for the
+    last layer's activations, the same bits as the default tiles."""
+    import torch
+    ddf, a, b = _pair(net, precision)
+    rays = _dev(torch, I.uniform_rays(n, seed=n))
+    want = b.query(rays)
+    for x, y in zip(a.query(rays), want):
+        assert torch.equal(x, y)
+    if n <= 5761:                        # the static scratch holds 6,061 rays of the widest
+        t, v = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+        ddf.ddf_query_rays_noalloc(a.h, rays, n, t, v, torch.cuda.current_stream())
+        assert torch.equal(t, want[0]) and torch.equal(v, want[1])
+    assert ddf.ddf_check_status(a.h) == 0
+
+
+@pytest.mark.parametrize("net,precision,n", [((4, 768, 2), "bf16", 38911), ((4, 768, 2), "bf16", 38912),
+                                             ((4, 768, 2), "fp8", 64853), ((4, 768, 2), "fp8", 64854),
+                                             ((4, 384, 2), "bf16", 70001), ((4, 768, 1), "bf16", 896)])
+def test_the_line_of_the_pair_tiles(cuda_lib, net, precision, n):
+    """Six waves of wide tiles on 152 SMs (e4m3 ten); fields without pair tiles
+    have no such line; a single layer."""
+    import torch
+    ddf, a, b = _pair(net, precision)
+    rays = _dev(torch, I.uniform_rays(n, seed=5))
+    for x, y in zip(a.shadow(rays, LIGHT), b.shadow(rays, LIGHT)):
+        assert torch.equal(x, y)
+    assert ddf.ddf_check_status(a.h) == 0
