@@ -123,6 +123,7 @@ void release_weight_buffers(ddf_s* h) {
   h->tmSmall.clear();
   h->tmTrace.clear();
   h->tmStep.clear();
+  h->tmF32.clear();
   h->wcal.clear();
   h->wp.clear();
   h->wq.clear();
@@ -289,8 +290,6 @@ ddf_status forward_f32_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, c
     DDF_CK(ddf::launch_encode_planes(rays, m, h->cfg.octaves, h->kp32,
                                      static_cast<__nv_bfloat16*>(h->ws_enc), st));
   }
-  const int64_t tiles = ((m + 255) / 256) * static_cast<int64_t>(W / 256);
-  const int clusters = static_cast<int>(std::min<int64_t>(tiles, h->f32_clusters));
   for (int l = 0; l < H; ++l) {
     const void* a_base = l == 0 ? h->ws_enc : h->ws_act[(l - 1) & 1];
     ddf::TcF32Params p{};
@@ -309,7 +308,7 @@ ddf_status forward_f32_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, c
                    static_cast<uint64_t>(p.K) * 2, 128))
       return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation map");
     ProfScope ps(h, l == 0 ? kProfFirst : kProfGemm, st);
-    DDF_CK(ddf::launch_tc_gemm_f32(tmA, h->tmB[l], p, clusters, st));
+    DDF_CK(ddf::launch_tc_gemm_f32(tmA, h->tmB[l], h->tmF32[l], p, h->f32_clusters, st));
   }
   ProfScope ps(h, kProfHead, st);
   DDF_CK(ddf::launch_head_f32(static_cast<const float*>(h->ws_act[(H - 1) & 1]), m, W, h->head_w,
@@ -1109,6 +1108,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     h->wcal.assign(H, nullptr);
     h->tmB.assign(H, CUtensorMap{});
     h->tmBcal.assign(H, CUtensorMap{});
+    h->tmF32.assign(H, CUtensorMap{});
     std::vector<CUtensorMap> narrow(h->narrow ? H : 0);
     for (int l = 0; l < H; ++l) {
       const int K = l == 0 ? h->d_in : W;
@@ -1123,8 +1123,9 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
         } else {
           if ((s = dev_alloc(h, &p, static_cast<size_t>(W) * kp * 6)) != DDF_OK) return s;
           h->wp[l] = static_cast<__nv_bfloat16*>(p);
-          if (!make_tmap(&h->tmB[l], h->wp[l], false, kp, 3 * static_cast<uint64_t>(W),
-                         static_cast<uint64_t>(kp) * 2, 128))
+          const uint64_t rows = 3 * static_cast<uint64_t>(W), pitch = static_cast<uint64_t>(kp) * 2;
+          if (!make_tmap(&h->tmB[l], h->wp[l], false, kp, rows, pitch, 128) ||
+              !make_tmap(&h->tmF32[l], h->wp[l], false, kp, rows, pitch, 32))
             return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
         }
       } else if (prec == DDF_BF16 || l == 0) {

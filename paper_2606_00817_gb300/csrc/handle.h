@@ -59,6 +59,7 @@ struct ddf_s {
   int f32_clusters = 0;
   int64_t f32_pass = 131072;
   std::vector<__nv_bfloat16*> wp;
+  std::vector<CUtensorMap> tmF32;  // its maps with boxes of 32 rows (tmB: 128)
   std::vector<float*> bias;  // per hidden layer [W]
   std::vector<__nv_bfloat16*> wb;  // bf16 W (all layers for BF16, layer 1 for FP8)
   std::vector<uint8_t*> wq;        // FP8: e4m3 codes for layers 2..H

@@ -219,8 +219,8 @@ cudaError_t launch_sgemm_relu(const float* A, const float* W, const float* b, fl
 
 // FP32 layer on the tensor cores (tc_gemm_f32.cu): ReLU(A W^T + b) with both
 // operands given as three bf16 planes that add up to the FP32 values. tmA maps
-// A's planes as one [3 M x K] matrix, tmB W's as [3 N x K], with 128-row boxes;
-// N % 256 == 0. The output is either the next layer's planes [3][M x N] or
+// A's planes as one [3 M x K] matrix, tmB W's as [3 N x K], with 128-row boxes, tmB32
+// the same with 32-row boxes; N % 256 == 0; clusters: as many as the GPU holds. The output is either the next layer's planes [3][M x N] or
 // FP32 rows [M x N]; both and bias 16-byte aligned.
 struct TcF32Params {
   int M, N, K;
@@ -231,7 +231,8 @@ struct TcF32Params {
   uint64_t timeout_ns;
 };
 cudaError_t launch_tc_gemm_f32(const CUtensorMap& tmA, const CUtensorMap& tmB,
-                               const TcF32Params& p, int clusters, cudaStream_t s);
+                               const CUtensorMap& tmB32, const TcF32Params& p, int clusters,
+                               cudaStream_t s);
 int tc_gemm_f32_max_clusters();
 // The encoded rays as planes [3][M x ld], and the planes [3][N x ldd] of
 // src [N x K] zero-padded to ldd columns (a multiple of 8).

@@ -8,9 +8,9 @@
 // 2^-26 of |a w| each, and of random sign (the pieces are rounded to nearest).
 //
 // What bounds it: the tensor pipe, at six bf16 MMAs per FP32 one. Measured
-// through the 126 -> 1280 x 8 field: 16,387 rays 1.88 ms against 9.53 ms on
-// FFMA (sgemm_relu_kernel), 1 ray 0.34 against 1.40 ms; at 256 x 3, 5,000
-// rays 0.088 against 0.128 ms. It wins at every batch size, so a width that is
+// through the 126 -> 1280 x 8 field: 16,387 rays 1.80 ms against 9.54 ms on
+// FFMA (sgemm_relu_kernel), 1 ray 0.24 against 1.40 ms; at 256 x 3, 5,000
+// rays 0.06 against 0.128 ms. It wins at every batch size, so a width that is
 // a multiple of 256 always takes it; other widths keep the FFMA layers.
 //
 // Precision. The MMA adds into its FP32 accumulator without rounding to
@@ -56,9 +56,94 @@ static_assert(kF32Smem <= 227 * 1024, "shared memory of one CTA");
 __device__ constexpr int kProdA[6] = {2, 0, 1, 1, 0, 0};
 __device__ constexpr int kProdW[6] = {0, 2, 1, 0, 1, 0};
 
+// The tiles of a layer on `slots` clusters: whole waves of 256 x 256 tiles, and
+// each tile left over in 1 << lg parts of 256 >> lg columns, as many as one wave
+// holds (a part of 64 columns takes a third of a tile's time, by its operands).
+// 1280 x 8, undivided and so: 1 ray (5 tiles of 76) 337 and 243 us, 1,000 rays (20)
+// 406 and 314, 4,099 rays (a wave and 9) 739 and 609, 16,387 rays 1,880 and 1,800.
+struct F32Plan {
+  int big, lg, tiles;
+};
+__host__ __device__ inline F32Plan f32_plan(int M, int N, int slots) {
+  const int all = (M + 255) / 256 * (N / 256), big = all / slots * slots, rest = all - big;
+  const int lg = 4 * rest <= slots ? 2 : 2 * rest <= slots ? 1 : 0;
+  return F32Plan{big, lg, big + (rest << lg)};
+}
+struct F32Tile {
+  int m0, n0, n;  // first row and column, columns
+};
+__device__ __forceinline__ F32Tile f32_tile(const F32Plan& f, int t, int num_n) {
+  int sub = 0, n = 256;
+  if (t >= f.big) {
+    const int u = t - f.big;
+    sub = u & ((1 << f.lg) - 1);
+    t = f.big + (u >> f.lg);
+    n = 256 >> f.lg;
+  }
+  return F32Tile{t / num_n * 256, t % num_n * 256 + sub * n, n};
+}
+
+// One warp's part of a tile: COLS columns of its 32 rows, the accumulators of
+// every 32 of K added up (`it` counts them), then bias, ReLU and the output at the
+// row and column `where` gives (asked late: its registers are not there before).
+// False when a wait gave up.
+template <int COLS, class Wait, class Done, class Where>
+__device__ __forceinline__ bool f32_drain(const TcF32Params& p, uint32_t trow, int blocks,
+                                          uint32_t& it, Wait wait, Done done, Where where) {
+  float acc[COLS];
+#pragma unroll
+  for (int i = 0; i < COLS; ++i) acc[i] = 0.f;
+  for (int kb = 0; kb < blocks; ++kb, ++it) {
+    const int b = it & 1;
+    if (!wait(b, (it >> 1) & 1)) return false;
+    tc_fence_after();
+#pragma unroll
+    for (int c = 0; c < COLS / 16; ++c) {  // 16 columns at a time: 32 would spill
+      uint32_t v[16];
+      tmem_ld16_wait(trow + 256u * b + 16u * c, v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) acc[16 * c + i] += __uint_as_float(v[i]);
+    }
+    tc_fence_before();
+    __syncwarp();
+    done(b);
+  }
+  int row, n0;
+  where(row, n0);
+  if (row >= p.M) return true;
+  const float4* bias = reinterpret_cast<const float4*>(p.bias + n0);
+#pragma unroll
+  for (int c = 0; c < COLS / 4; ++c) {
+    const float4 bb = __ldg(bias + c);
+    acc[4 * c + 0] = fmaxf(acc[4 * c + 0] + bb.x, 0.f);
+    acc[4 * c + 1] = fmaxf(acc[4 * c + 1] + bb.y, 0.f);
+    acc[4 * c + 2] = fmaxf(acc[4 * c + 2] + bb.z, 0.f);
+    acc[4 * c + 3] = fmaxf(acc[4 * c + 3] + bb.w, 0.f);
+  }
+  if (p.out_f32 != nullptr) {  // the last layer: FP32 rows for the head
+    float4* dst = reinterpret_cast<float4*>(p.out_f32 + static_cast<size_t>(row) * p.N + n0);
+#pragma unroll
+    for (int c = 0; c < COLS / 4; ++c)
+      dst[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+  } else {  // the next layer's operand: three bf16 planes
+#pragma unroll
+    for (int c = 0; c < COLS / 8; ++c) {
+      uint4 w[3];
+      f32_split8(acc + 8 * c, w);
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        *reinterpret_cast<uint4*>(p.out_planes +
+                                  (static_cast<size_t>(j) * p.M + row) * p.N + n0 + 8 * c) = w[j];
+    }
+  }
+  return true;
+}
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
     tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA,
-                       const __grid_constant__ CUtensorMap tmB, const TcF32Params p) {
+                       const __grid_constant__ CUtensorMap tmB,
+                       const __grid_constant__ CUtensorMap tmB32, const TcF32Params p,
+                       const int slots) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -111,16 +196,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
   };
 
   const int num_n = p.N / 256;
-  const int num_tiles = ((p.M + 255) / 256) * num_n;
+  const F32Plan plan = f32_plan(p.M, p.N, slots);
+  const int num_tiles = plan.tiles;
   const int num_kb = (p.K + 63) / 64;
-  // plane j of A starts at row j M of the map, plane j of W at row j N
-  auto load_stage = [&](int s, int m0, int n0, int kb, uint32_t bar) {
+  // plane j of A starts at row j M of the map, plane j of W at row j N; this CTA
+  // brings 128 rows of A and half of the tile's rows of W
+  auto load_stage = [&](int s, const F32Tile& t, int kb, uint32_t bar) {
     const uint32_t a = smem_u32(smem + s * kF32Stage);
+    const int m0 = t.m0 + static_cast<int>(rank) * 128, n0 = t.n0 + static_cast<int>(rank) * (t.n / 2);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       tma_load_2d_pair(a + j * kF32Plane, &tmA, kb * 64, j * p.M + m0, bar);
-      tma_load_2d_pair(a + kF32Operand + j * kF32Plane, &tmB, kb * 64, j * p.N + n0, bar);
+      const uint32_t b = a + kF32Operand + j * kF32Plane;
+      if (t.n == 256) {
+        tma_load_2d_pair(b, &tmB, kb * 64, j * p.N + n0, bar);
+      } else {
+        for (int r = 0; r < t.n / 2; r += 32)
+          tma_load_2d_pair(b + r * 128, &tmB32, kb * 64, j * p.N + n0 + r, bar);
+      }
     }
+  };
+  auto stage_bytes = [](const F32Tile& t) {  // of both CTAs
+    return static_cast<uint32_t>(2 * (kF32Operand + 3 * (t.n / 2) * 128));
   };
 
   if (warp == 0) {
@@ -129,16 +226,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        const int m0 = (tile / num_n) * 256 + static_cast<int>(rank) * 128;
-        const int n0 = (tile % num_n) * 256 + static_cast<int>(rank) * 128;
+        const F32Tile t = f32_tile(plan, tile, num_n);
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it & 1;
           if (!mbar_wait_bounded(empty_bar(s), ((it >> 1) & 1) ^ 1u, abort_flag, p.timeout_ns)) {
             ok = false;
             break;
           }
-          if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * kF32Stage);
-          load_stage(s, m0, n0, kb, full_leader0 + 8u * s);
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(s), stage_bytes(t));
+          load_stage(s, t, kb, full_leader0 + 8u * s);
         }
       }
       if (!ok) raise_abort();
@@ -149,10 +245,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       // -------------------------------------------------------- MMA issuer
-      constexpr uint32_t idesc = mma_idesc(1u, 256, 256);
       uint32_t it = 0;  // one K block: one stage and one accumulator
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
+        const uint32_t idesc = mma_idesc(1u, f32_tile(plan, tile, num_n).n, 256);
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it & 1;
           const uint32_t ph = (it >> 1) & 1;
@@ -187,66 +283,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
   } else {
     // ---------------------------------------------------------- epilogue (both CTAs)
     const int q = warp & 3;            // TMEM lane quarter
-    const int half = (warp - 2) / 4;   // columns [128 half, 128 half + 128)
+    const int half = (warp - 2) / 4;   // half of the tile's columns
     const uint32_t tempty_leader0 = map_to_cta(tempty_bar(0), 0);
-    const uint32_t trow = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + 128u * half;
+    const uint32_t trow = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+    auto wait = [&](int b, uint32_t ph) {
+      const bool ok = mbar_wait_bounded(tfull_bar(b), ph, abort_flag, p.timeout_ns);
+      return __all_sync(0xffffffffu, ok) != 0;
+    };
+    auto done = [&](int b) {
+      if (lane == 0) mbar_arrive_cluster(tempty_leader0 + 8u * b);
+    };
     uint32_t it = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-      float acc[128];
-#pragma unroll
-      for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-      for (int kb = 0; kb < 2 * num_kb; ++kb, ++it) {
-        const int b = it & 1;
-        ok = mbar_wait_bounded(tfull_bar(b), (it >> 1) & 1, abort_flag, p.timeout_ns);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) {
-          if (lane == 0) raise_abort();
-          break;
-        }
-        tc_fence_after();
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {  // 16 columns at a time: 32 would spill
-          uint32_t v[16];
-          tmem_ld16_wait(trow + 256u * b + 16u * c, v);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) acc[16 * c + i] += __uint_as_float(v[i]);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(tempty_leader0 + 8u * b);
-      }
-      if (!ok) break;
-      const int row = (tile / num_n) * 256 + static_cast<int>(rank) * 128 + q * 32 + lane;
-      const int n0 = (tile % num_n) * 256 + 128 * half;
-      if (row >= p.M) continue;
-      const float4* bias = reinterpret_cast<const float4*>(p.bias + n0);
-#pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        const float4 bb = __ldg(bias + c);
-        acc[4 * c + 0] = fmaxf(acc[4 * c + 0] + bb.x, 0.f);
-        acc[4 * c + 1] = fmaxf(acc[4 * c + 1] + bb.y, 0.f);
-        acc[4 * c + 2] = fmaxf(acc[4 * c + 2] + bb.z, 0.f);
-        acc[4 * c + 3] = fmaxf(acc[4 * c + 3] + bb.w, 0.f);
-      }
-      if (p.out_f32 != nullptr) {  // the last layer: FP32 rows for the head
-        float4* dst = reinterpret_cast<float4*>(p.out_f32 + static_cast<size_t>(row) * p.N + n0);
-#pragma unroll
-        for (int c = 0; c < 32; ++c)
-          dst[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
-      } else {  // the next layer's operand: three bf16 planes
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          uint4 w[3];
-          f32_split8(acc + 8 * c, w);
-#pragma unroll
-          for (int j = 0; j < 3; ++j)
-            *reinterpret_cast<uint4*>(p.out_planes +
-                                      (static_cast<size_t>(j) * p.M + row) * p.N + n0 + 8 * c) =
-                w[j];
-        }
-      }
+      const int n = tile < plan.big ? 256 : 256 >> plan.lg;
+      auto where = [&](int& row, int& n0) {
+        const F32Tile t = f32_tile(f32_plan(p.M, p.N, slots), tile, p.N / 256);
+        row = t.m0 + static_cast<int>(rank) * 128 + q * 32 + lane;
+        n0 = t.n0 + t.n / 2 * half;
+      };
+      if (n == 256)
+        ok = f32_drain<128>(p, trow + 128u * half, 2 * num_kb, it, wait, done, where);
+      else if (n == 128)
+        ok = f32_drain<64>(p, trow + 64u * half, 2 * num_kb, it, wait, done, where);
+      else
+        ok = f32_drain<32>(p, trow + 32u * half, 2 * num_kb, it, wait, done, where);
     }
+    if (!ok && lane == 0) raise_abort();
   }
 
   // ---------------------------------------------------------- teardown
@@ -256,9 +319,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
     const uint32_t mine = issued[rank], other = issued[rank ^ 1u];
     // after an abort: copy this CTA's half of any stage the other producer
     // issued and this one did not, so that every armed phase completes
-    for (uint32_t j = mine; j < other; ++j) {
-      if (rank == 0) mbar_arrive_expect_tx(full_bar(j & 1), 2 * kF32Stage);
-      load_stage(j & 1, 0, 0, 0, full_leader0 + 8u * (j & 1));
+    for (uint32_t j = mine; j < other; ++j) {  // K block j of this pair's tiles
+      const F32Tile t =
+          f32_tile(plan, pair + static_cast<int>(j / num_kb) * npairs, num_n);
+      if (rank == 0) mbar_arrive_expect_tx(full_bar(j & 1), stage_bytes(t));
+      load_stage(j & 1, t, static_cast<int>(j % num_kb), full_leader0 + 8u * (j & 1));
     }
     if (rank == 0) {
       const uint32_t jmax = mine > other ? mine : other;
@@ -314,7 +379,8 @@ int tc_gemm_f32_max_clusters() {
 }
 
 cudaError_t launch_tc_gemm_f32(const CUtensorMap& tmA, const CUtensorMap& tmB,
-                               const TcF32Params& p, int clusters, cudaStream_t s) {
+                               const CUtensorMap& tmB32, const TcF32Params& p, int clusters,
+                               cudaStream_t s) {
   if (p.M <= 0) return cudaSuccess;
   if (p.N % 256 != 0 || p.K <= 0 || clusters <= 0 ||
       3 * static_cast<int64_t>(p.M) > 0x7fffffff ||
@@ -326,7 +392,9 @@ cudaError_t launch_tc_gemm_f32(const CUtensorMap& tmA, const CUtensorMap& tmB,
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_f32_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, kF32Smem);
   if (e != cudaSuccess) return e;
-  tc_gemm_f32_kernel<<<2 * clusters, kF32Threads, kF32Smem, s>>>(tmA, tmB, p);
+  const int tiles = f32_plan(p.M, p.N, clusters).tiles;
+  tc_gemm_f32_kernel<<<2 * (tiles < clusters ? tiles : clusters), kF32Threads, kF32Smem, s>>>(
+      tmA, tmB, tmB32, p, clusters);
   return cudaGetLastError();
 }
 

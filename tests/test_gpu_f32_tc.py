@@ -76,3 +76,17 @@ def test_rows_that_are_not_finite_leave_the_others_alone(cuda_lib):
     # a NaN coordinate makes every pre-activation NaN, which the ReLU takes to
     # 0, so the row's outputs are those of zero activations in layer 2
     assert torch.isfinite(t[~keep][:1]).all()
+
+
+@pytest.mark.parametrize("n", [1, 256, 769, 1025, 2048, 3841, 4097, 5000])
+def test_whole_and_split_tiles_agree(cuda_lib, n):
+    """At width 1280 five tiles per 256 rows: batches of less than a wave of
+    them in four or two parts, a wave and a rest, and the last rows of a batch
+    of several waves: the same bits."""
+    import torch
+    ddf, m, _ = _field((4, 1280, 2))
+    rays = _dev(torch, I.uniform_rays(16387, seed=6))
+    t, v = m.query(rays)
+    a, b = m.query([r[-n:].clone() for r in rays])
+    assert torch.equal(a, t[-n:]) and torch.equal(b, v[-n:])
+    assert ddf.ddf_check_status(m.h) == 0
