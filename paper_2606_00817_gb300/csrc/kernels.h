@@ -221,7 +221,7 @@ cudaError_t launch_sgemm_relu(const float* A, const float* W, const float* b, fl
 // operands given as three bf16 planes that add up to the FP32 values. tmA maps
 // A's planes as one [3 M x K] matrix, tmB W's as [3 N x K], with 128-row boxes, tmB32
 // the same with 32-row boxes; N % 256 == 0; clusters: as many as the GPU holds. The output is either the next layer's planes [3][M x N] or
-// FP32 rows [M x N]; both and bias 16-byte aligned.
+// FP32 rows [M x N], 32-byte aligned; bias 16-byte aligned.
 struct TcF32Params {
   int M, N, K;
   const float* bias;

@@ -7,11 +7,15 @@
 // of bf16 operands, each exact in FP32. The three products left out are below
 // 2^-26 of |a w| each, and of random sign (the pieces are rounded to nearest).
 //
-// What bounds it: the tensor pipe, at six bf16 MMAs per FP32 one. Measured
-// through the 126 -> 1280 x 8 field: 16,387 rays 1.80 ms against 9.54 ms on
-// FFMA (sgemm_relu_kernel), 1 ray 0.24 against 1.40 ms; at 256 x 3, 5,000
-// rays 0.06 against 0.128 ms. It wins at every batch size, so a width that is
-// a multiple of 256 always takes it; other widths keep the FFMA layers.
+// What bounds it: the tensor pipe, at six bf16 MMAs per FP32 one, and between
+// two tiles the outputs (the epilogue warps hold a tile's sums in registers, so
+// the MMAs run at most two accumulators ahead of them). Measured through the
+// 126 -> 1280 x 8 field: 16,387 rays 1.53 ms against 9.53 ms on FFMA
+// (sgemm_relu_kernel), without any output stores 1.18, without operand loads or
+// without reading the accumulators no less; 140,000 rays 11.8 ms, 1 ray 0.24
+// against 1.40 ms; at 256 x 3, 5,000 rays 0.06 against 0.128 ms. It wins at every
+// batch size, so a width that is a multiple of 256 always takes it; other widths
+// keep the FFMA layers.
 //
 // Precision. The MMA adds into its FP32 accumulator without rounding to
 // nearest, so a long sum in TMEM would drift. An accumulator therefore only
@@ -33,6 +37,7 @@
 // Waits are bounded and an abort drains as in the pair kernel.
 #include <cuda_bf16.h>
 
+#include "epilogue.cuh"
 #include "f32_split.cuh"
 #include "kernels.h"
 #include "ptx_sm103.cuh"
@@ -60,27 +65,30 @@ __device__ constexpr int kProdW[6] = {0, 2, 1, 0, 1, 0};
 // each tile left over in 1 << lg parts of 256 >> lg columns, as many as one wave
 // holds (a part of 64 columns takes a third of a tile's time, by its operands).
 // 1280 x 8, undivided and so: 1 ray (5 tiles of 76) 337 and 243 us, 1,000 rays (20)
-// 406 and 314, 4,099 rays (a wave and 9) 739 and 609, 16,387 rays 1,880 and 1,800.
+// 406 and 314, 4,099 rays (a wave and 9) 739 and 609.
+// The parts come first: the clusters that begin with one are out of step with the
+// others from then on, and their outputs' stores do not all fall together (1,506 and
+// 1,484 us).
 struct F32Plan {
-  int big, lg, tiles;
+  int parts, lg, tiles;
 };
 __host__ __device__ inline F32Plan f32_plan(int M, int N, int slots) {
   const int all = (M + 255) / 256 * (N / 256), big = all / slots * slots, rest = all - big;
   const int lg = 4 * rest <= slots ? 2 : 2 * rest <= slots ? 1 : 0;
-  return F32Plan{big, lg, big + (rest << lg)};
+  return F32Plan{rest << lg, lg, big + (rest << lg)};
 }
 struct F32Tile {
   int m0, n0, n;  // first row and column, columns
 };
+__device__ __forceinline__ int f32_columns(const F32Plan& f, int t) {
+  return t < f.parts ? 256 >> f.lg : 256;
+}
 __device__ __forceinline__ F32Tile f32_tile(const F32Plan& f, int t, int num_n) {
-  int sub = 0, n = 256;
-  if (t >= f.big) {
-    const int u = t - f.big;
-    sub = u & ((1 << f.lg) - 1);
-    t = f.big + (u >> f.lg);
-    n = 256 >> f.lg;
-  }
-  return F32Tile{t / num_n * 256, t % num_n * 256 + sub * n, n};
+  const int n = f32_columns(f, t);
+  const int sub = t < f.parts ? t & ((1 << f.lg) - 1) : 0;
+  t = t < f.parts ? t >> f.lg : t - f.parts + (f.parts >> f.lg);
+  const int m = t / num_n;
+  return F32Tile{m * 256, (t - m * num_n) * 256 + sub * n, n};
 }
 
 // One warp's part of a tile: COLS columns of its 32 rows, the accumulators of
@@ -120,20 +128,30 @@ __device__ __forceinline__ bool f32_drain(const TcF32Params& p, uint32_t trow, i
     acc[4 * c + 2] = fmaxf(acc[4 * c + 2] + bb.z, 0.f);
     acc[4 * c + 3] = fmaxf(acc[4 * c + 3] + bb.w, 0.f);
   }
+  // 32-byte stores: the lanes' rows lie apart, and with half-written sectors this
+  // part took a third of a layer's time (16,387 rays 1.80 ms, now 1.53; TMA stores
+  // from shared-memory boxes, for which only 32 KB are left, 1.69)
   if (p.out_f32 != nullptr) {  // the last layer: FP32 rows for the head
-    float4* dst = reinterpret_cast<float4*>(p.out_f32 + static_cast<size_t>(row) * p.N + n0);
-#pragma unroll
-    for (int c = 0; c < COLS / 4; ++c)
-      dst[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
-  } else {  // the next layer's operand: three bf16 planes
+    float* dst = p.out_f32 + static_cast<size_t>(row) * p.N + n0;
 #pragma unroll
     for (int c = 0; c < COLS / 8; ++c) {
-      uint4 w[3];
-      f32_split8(acc + 8 * c, w);
+      uint32_t w[8];
 #pragma unroll
-      for (int j = 0; j < 3; ++j)
-        *reinterpret_cast<uint4*>(p.out_planes +
-                                  (static_cast<size_t>(j) * p.M + row) * p.N + n0 + 8 * c) = w[j];
+      for (int i = 0; i < 8; ++i) w[i] = __float_as_uint(acc[8 * c + i]);
+      st_global_256(dst + 8 * c, w);
+    }
+  } else {  // the next layer's operand: three bf16 planes
+#pragma unroll
+    for (int c = 0; c < COLS / 16; ++c) {
+      uint4 lo[3], hi[3];
+      f32_split8(acc + 16 * c, lo);
+      f32_split8(acc + 16 * c + 8, hi);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const uint32_t w[8] = {lo[j].x, lo[j].y, lo[j].z, lo[j].w,
+                               hi[j].x, hi[j].y, hi[j].z, hi[j].w};
+        st_global_256(p.out_planes + (static_cast<size_t>(j) * p.M + row) * p.N + n0 + 16 * c, w);
+      }
     }
   }
   return true;
@@ -248,7 +266,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
       uint32_t it = 0;  // one K block: one stage and one accumulator
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        const uint32_t idesc = mma_idesc(1u, f32_tile(plan, tile, num_n).n, 256);
+        const uint32_t idesc = mma_idesc(1u, f32_columns(plan, tile), 256);
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it & 1;
           const uint32_t ph = (it >> 1) & 1;
@@ -296,7 +314,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
     uint32_t it = 0;
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-      const int n = tile < plan.big ? 256 : 256 >> plan.lg;
+      const int n = f32_columns(plan, tile);
       auto where = [&](int& row, int& n0) {
         const F32Tile t = f32_tile(f32_plan(p.M, p.N, slots), tile, p.N / 256);
         row = t.m0 + static_cast<int>(rank) * 128 + q * 32 + lane;
@@ -385,8 +403,8 @@ cudaError_t launch_tc_gemm_f32(const CUtensorMap& tmA, const CUtensorMap& tmB,
   if (p.N % 256 != 0 || p.K <= 0 || clusters <= 0 ||
       3 * static_cast<int64_t>(p.M) > 0x7fffffff ||
       (p.out_f32 == nullptr) == (p.out_planes == nullptr) ||
-      reinterpret_cast<uintptr_t>(p.out_f32) % 16 != 0 ||
-      reinterpret_cast<uintptr_t>(p.out_planes) % 16 != 0 ||
+      reinterpret_cast<uintptr_t>(p.out_f32) % 32 != 0 ||
+      reinterpret_cast<uintptr_t>(p.out_planes) % 32 != 0 ||
       reinterpret_cast<uintptr_t>(p.bias) % 16 != 0)
     return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_f32_kernel,
