@@ -544,8 +544,13 @@ typedef struct {
 } ddf_tile;
 
 /* Tile of layer 1 (which = 1) or of layers 2..H (which = 0). Results agree
- * across tiles up to FP32 rounding of the head sums. Default: bn 256 where
- * possible, 4 warps, no pair, not staged, for both. Synchronises the device
+ * across tiles up to FP32 rounding of the head sums. Until one is set,
+ * ddf_get_tile reports bn 256 where possible, 4 warps, no pair, not staged, for
+ * both, and every batch takes the kernels that suit its size, with the results
+ * of that tile bit for bit: a width of 128 or 256 (bf16) one kernel for the whole
+ * query; else narrower tiles for small batches, whole and split tiles for
+ * middling ones, the pair tile and the fused layer 1 for large ones. A tile set
+ * here, or picked by ddf_autotune, holds for every batch. Synchronises the device
  * when weights are loaded. */
 ddf_status ddf_set_tile(ddf_handle h, int32_t which, const ddf_tile* tile);
 ddf_status ddf_get_tile(ddf_handle h, int32_t which, ddf_tile* tile);
@@ -561,7 +566,8 @@ ddf_status ddf_get_tile(ddf_handle h, int32_t which, ddf_tile* tile);
  * over 3 rounds, one query each, and keep their best round (so a clock that
  * drifts under the power cap affects all alike): phase 1 times every launch
  * of the query, phase 2 the encoding and layer-1 launches only (CUDA events
- * around each launch). ms_out (nullable,
+ * around each launch). A bf16 field of width 128 or 256 keeps its one kernel
+ * where none of the tiles is faster. ms_out (nullable,
  * n_out >= 18) receives the per-query ms of phase 1 in [0..8] (7, 8 unused)
  * and of phase 2 in [9..17], -1 where a candidate was skipped or rejected.
  * Synchronous; allocates 16 n bytes of device memory while it runs. A no-op

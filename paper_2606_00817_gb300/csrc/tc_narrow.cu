@@ -14,9 +14,10 @@
 //     side by side where there is room, one in its MMAs while the other drains;
 //   * streamed: a ring of chunks, refilled as the MMAs release them, so the
 //     next layer's weights arrive while a layer drains. One group.
-// Measured, a whole call: 78 -> 128 x 4, 16,384 rays 42 us by layers, 32 us so (both
-// near the host cost of a call), 300,000 rays 166 and 114 us; 102 -> 256 x 3, 100,000
-// rays 102 and 85 us, 1,000,000 rays 708 and 677 us. It wins at every size measured.
+// Measured, a whole call: 78 -> 128 x 4, 16,384 rays 42 us by layers, 22 us so (near
+// the host cost of a call), 300,000 rays 166 and 101 us; 102 -> 256 x 3, 100,000
+// rays 102 and 73 us, 300,000 rays 241 and 185, 1,000,000 rays 708 and 585 us. It wins
+// at every size measured.
 //
 // The arithmetic is that of the layer kernels, in their order (encode_kernel,
 // K ascending in steps of 16, ReLU(acc + b) rounded to bf16, the head's FP32
