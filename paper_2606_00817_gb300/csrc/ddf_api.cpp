@@ -130,8 +130,6 @@ void release_weight_buffers(ddf_s* h) {
   dev_free(h, h->head_w);
   dev_free(h, h->head_b);
   dev_free(h, h->d_blob);
-  dev_free(h, h->narrow_maps);
-  h->narrow_maps = nullptr;
   h->head_w = h->head_b = h->d_blob = nullptr;
   h->loaded = false;
 }
@@ -438,14 +436,13 @@ ddf_status forward_tc(ddf_s* h, ddf::RaySoA rays, int m, ddf::HeadOut out, cudaS
     p.M = m;
     p.L = h->cfg.octaves;
     p.H = H;
-    p.maps = h->narrow_maps;
     for (int l = 0; l < H; ++l) p.bias[l] = h->bias[l];
     p.head_w = h->head_w;
     p.head_b = h->head_b;
     p.status = h->status_dev;
     p.timeout_ns = h->timeout_ns;
     ProfScope ps(h, kProfGemm, st);
-    DDF_CK(ddf::launch_tc_narrow(p, rays, out, W, h->num_sms, st));
+    DDF_CK(ddf::launch_tc_narrow(h->narrow_maps, p, rays, out, W, h->num_sms, st));
     return DDF_OK;
   }
   if (h->tile_auto && !h->tmSmall.empty() && m <= small_rows(W, h->num_sms) && m <= h->ws_x_rows)
@@ -1109,7 +1106,6 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
     h->tmB.assign(H, CUtensorMap{});
     h->tmBcal.assign(H, CUtensorMap{});
     h->tmF32.assign(H, CUtensorMap{});
-    std::vector<CUtensorMap> narrow(h->narrow ? H : 0);
     for (int l = 0; l < H; ++l) {
       const int K = l == 0 ? h->d_in : W;
       if ((s = dev_alloc(h, &p, W * sizeof(float))) != DDF_OK) return s;
@@ -1135,7 +1131,7 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
         if (!make_tmap(&h->tmB[l], h->wb[l], false, kp, W, static_cast<uint64_t>(kp) * 2,
                        (l == 0 ? h->tile_first : h->tile).pair ? 128u : (l == 0 ? h->tile_first : h->tile).bn))
           return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
-        if (h->narrow && !make_tmap(&narrow[l], h->wb[l], false, kp, W,
+        if (h->narrow && !make_tmap(&h->narrow_maps.m[l], h->wb[l], false, kp, W,
                                     static_cast<uint64_t>(kp) * 2, static_cast<uint32_t>(W)))
           return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
       } else {
@@ -1160,11 +1156,6 @@ ddf_status ddf_load_weights(ddf_handle h, const float* host_blob, size_t n_float
         if (!make_tmap(&h->tmBcal[l], w, false, kp, W, static_cast<uint64_t>(kp) * 2, h->bn))
           return fail(DDF_ERR_CUDA, "cuTensorMapEncodeTiled failed for a weight map");
       }
-    }
-    if (h->narrow) {
-      if ((s = dev_alloc(h, &p, H * sizeof(CUtensorMap))) != DDF_OK) return s;
-      h->narrow_maps = static_cast<CUtensorMap*>(p);
-      DDF_CK(cudaMemcpy(p, narrow.data(), H * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
     }
     if ((s = dev_alloc(h, &p, 2 * W * sizeof(float))) != DDF_OK) return s;
     h->head_w = static_cast<float*>(p);

@@ -41,7 +41,7 @@ struct ddf_s {
   bool tile_auto = true;
   std::vector<CUtensorMap> tmSmall;  // weight maps of the small-batch tile
   std::vector<CUtensorMap> tmBig;  // weight maps of the tiles that large batches take by themselves
-  CUtensorMap* narrow_maps = nullptr;  // device: a launch does not carry 2 KB of maps
+  ddf::NarrowMaps narrow_maps{};  // weight maps of the one-kernel query
   int pair_clusters = 0;  // co-resident clusters of the CTA-pair kernel
   int num_sms = 0;
   bool loaded = false;

@@ -245,9 +245,14 @@ cudaError_t launch_pack_planes(const float* src, int N, int K, int ldd, __nv_bfl
 // 128 or 256, 1 .. kNarrowLayers hidden layers, every weight matrix mapped with
 // boxes of 64 K x `width` rows. The same bits as the default layer tiles.
 constexpr int kNarrowLayers = 16;
+// Passed by value, as a kernel parameter: a map in global memory would need an
+// acquire of the tensor-map proxy in every block before its first use, or a map
+// written later to the same address might not be seen.
+struct NarrowMaps {
+  CUtensorMap m[kNarrowLayers];  // one per layer
+};
 struct NarrowParams {
   int M, L, H;
-  const CUtensorMap* maps;  // device memory, one per layer
   const float* bias[kNarrowLayers];
   const float* head_w;  // [2 x width]
   const float* head_b;  // [2]
@@ -256,8 +261,8 @@ struct NarrowParams {
 };
 struct HeadOut;
 bool tc_narrow_supported(int L, int W, int H);
-cudaError_t launch_tc_narrow(const NarrowParams& p, const RaySoA& rays, const HeadOut& out,
-                             int W, int num_sms, cudaStream_t st);
+cudaError_t launch_tc_narrow(const NarrowMaps& maps, const NarrowParams& p, const RaySoA& rays,
+                             const HeadOut& out, int W, int num_sms, cudaStream_t st);
 
 // Heads: z = Wo h + bo, t = softplus(z0), vis = sigmoid(z1), optional shadow.
 struct HeadOut {

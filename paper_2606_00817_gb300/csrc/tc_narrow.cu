@@ -81,8 +81,9 @@ NwShape nw_shape(int L, int W, int H) {
 
 template <int W>
 __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
-    tc_narrow_kernel(const __grid_constant__ NarrowParams p, const NwShape sh,
-                     const __grid_constant__ RaySoA rays, const __grid_constant__ HeadOut out) {
+    tc_narrow_kernel(const __grid_constant__ NarrowMaps maps, const __grid_constant__ NarrowParams p,
+                     const NwShape sh, const __grid_constant__ RaySoA rays,
+                     const __grid_constant__ HeadOut out) {
   constexpr int kChunk = W * 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
   uint32_t load_ph = 0;
   auto load_chunk = [&]() {
     mbar_arrive_expect_tx(full_bar(load_slot), kChunk);
-    tma_load_2d(smem_u32(ring + load_slot * kChunk), p.maps + load_layer, load_kb * 64, 0,
+    tma_load_2d(smem_u32(ring + load_slot * kChunk), &maps.m[load_layer], load_kb * 64, 0,
                 full_bar(load_slot));
     ++loaded;
     if (++load_slot == sh.slots) {
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
   };
   int64_t total = 0;  // chunks this CTA needs
   if (producer && lane == 0) {
-    for (int l = 0; l < p.H; ++l) tma_prefetch_desc(p.maps + l);
+    for (int l = 0; l < p.H; ++l) tma_prefetch_desc(&maps.m[l]);
     for (int s = 0; s < sh.slots; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
@@ -359,14 +360,14 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
 }
 
 template <int W>
-cudaError_t launch_w(const NarrowParams& p, const NwShape& s,
+cudaError_t launch_w(const NarrowMaps& maps, const NarrowParams& p, const NwShape& s,
                      const RaySoA& rays, const HeadOut& out, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(tc_narrow_kernel<W>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (p.M + 127) / 128;
   const int grid = static_cast<int>(tiles < num_sms ? tiles : num_sms);
-  tc_narrow_kernel<W><<<grid, s.groups * kNwGroup + 32, s.smem, st>>>(p, s, rays, out);
+  tc_narrow_kernel<W><<<grid, s.groups * kNwGroup + 32, s.smem, st>>>(maps, p, s, rays, out);
   return cudaGetLastError();
 }
 
@@ -376,13 +377,13 @@ bool tc_narrow_supported(int L, int W, int H) {
   return (W == 128 || W == 256) && H >= 1 && H <= kNarrowLayers && nw_shape(L, W, H).slots > 0;
 }
 
-cudaError_t launch_tc_narrow(const NarrowParams& p, const RaySoA& rays, const HeadOut& out, int W,
-                             int num_sms, cudaStream_t st) {
+cudaError_t launch_tc_narrow(const NarrowMaps& maps, const NarrowParams& p, const RaySoA& rays,
+                             const HeadOut& out, int W, int num_sms, cudaStream_t st) {
   if (p.M <= 0) return cudaSuccess;
   if (!tc_narrow_supported(p.L, W, p.H)) return cudaErrorInvalidValue;
   const NwShape s = nw_shape(p.L, W, p.H);
-  return W == 128 ? launch_w<128>(p, s, rays, out, num_sms, st)
-                  : launch_w<256>(p, s, rays, out, num_sms, st);
+  return W == 128 ? launch_w<128>(maps, p, s, rays, out, num_sms, st)
+                  : launch_w<256>(maps, p, s, rays, out, num_sms, st);
 }
 
 }  // namespace ddf
