@@ -182,6 +182,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
   const int pair = blockIdx.x >> 1;
   const int npairs = gridDim.x >> 1;
 
+  cluster_arrive_relaxed();  // this CTA has started
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(full_bar(s), 1);
@@ -197,6 +198,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
   }
+  cluster_wait();  // and so has the peer, with which warp 1 allocates TMEM
   if (warp == 1) {
     tmem_alloc_pair(smem_u32(tmem_slot), 512);
     tmem_relinquish_pair();

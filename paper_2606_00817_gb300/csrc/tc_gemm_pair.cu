@@ -115,6 +115,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * (2 + EPI), 1)
   const int pair = blockIdx.x >> 1;
   const int npairs = gridDim.x >> 1;
 
+  cluster_arrive_relaxed();  // this CTA has started
   if (threadIdx.x == 0) {
     for (int s = 0; s < S::STAGES; ++s) {
       mbar_init(full_bar(s), 1);
@@ -132,11 +133,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * (2 + EPI), 1)
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
   }
+  const EpiVectors ev = stage_epi_vectors(p, reinterpret_cast<float*>(smem + S::VEC_OFFSET));
+  cluster_wait();  // and so has the peer, with which warp 1 allocates TMEM
   if (warp == 1) {
     tmem_alloc_pair(smem_u32(tmem_slot), S::TMEM_COLS);  // collective with the peer's warp 1
     tmem_relinquish_pair();
   }
-  const EpiVectors ev = stage_epi_vectors(p, reinterpret_cast<float*>(smem + S::VEC_OFFSET));
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs initialised, TMEM allocated
   tc_fence_after();

@@ -279,10 +279,9 @@ __device__ __forceinline__ void add4(float4& a, const float4 b) {
 
 // BATCHED: the partials' loads of a thread in flight together, and single
 // elements where rows are not whole float4s (a hash grid's MLP gradients, 16,384
-// rays: 22 -> 14 us). Not beside the CTA-pair GEMMs of a layered field, where it
-// gained nothing and, at 64 registers a thread instead of 40, a training loop on
-// one of several GPUs stopped making progress once in a few hundred steps; with
-// the plain loop 10,000 steps ran through.
+// rays: 22 -> 14 us). A layered field's reductions run beside its GEMMs and gained
+// nothing from it (65,536 rays through 1280 x 8: the same step), so they keep the
+// plain loop, at 40 registers a thread instead of 64.
 constexpr int kRedBatch = 8;  // 16-byte loads in flight a thread
 
 template <bool BATCHED>

@@ -31,3 +31,20 @@ def test_tensor_maps_reach_kernels_by_value():
         for args in re.findall(r"__global__.*?\((.*?)\)\s*\{", text, flags=re.S):
             assert not re.search(r"CUtensorMap\s*\*", args), name
         assert not re.search(r"cudaMemcpy\w*\([^;]*CUtensorMap", text), name
+
+
+def test_pair_allocations_follow_a_cluster_barrier():
+    """An allocation of tensor memory for a CTA pair works on the peer too and
+    waits without a limit, so every kernel first passes a cluster barrier, which
+    shows that the peer has started."""
+    found = 0
+    for name, text in _sources("*.cu").items():
+        for kernel in re.split(r"__global__", text)[1:]:
+            at = kernel.find("tmem_alloc_pair(")
+            if at < 0:
+                continue
+            found += 1
+            before = kernel[:at]
+            assert "cluster_sync_all()" in before or (
+                0 <= before.find("cluster_arrive_relaxed()") < before.find("cluster_wait()")), name
+    assert found >= 2
