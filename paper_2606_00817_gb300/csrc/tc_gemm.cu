@@ -157,13 +157,12 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         }
       }
     }
-    if (!ok) {
-      raise_abort(abort_flag, p.status);
-      // let every copy still in flight land before the CTA may exit
-      const int first = it > S::STAGES ? it - S::STAGES : 0;
-      for (int j = first; j < it; ++j)
-        mbar_wait_bounded(full_bar(j % S::STAGES), (j / S::STAGES) & 1, nullptr, kDrainTimeoutNs);
-    }
+    if (!ok) raise_abort(abort_flag, p.status);
+    // every copy still in flight lands before the CTA may exit: the MMA thread
+    // may have given up on them after this one had issued its last
+    const int first = it > S::STAGES ? it - S::STAGES : 0;
+    for (int j = first; j < it; ++j)
+      mbar_wait_bounded(full_bar(j % S::STAGES), (j / S::STAGES) & 1, nullptr, kDrainTimeoutNs);
   } else if (warp == 1 && lane == 0) {
     // ---------------------------------------------------------- MMA issuer
     constexpr uint32_t idesc_k = mma_idesc(IN_FP8 ? 0u : 1u, BN, S::BM);

@@ -162,12 +162,11 @@ __global__ void __launch_bounds__(64 + 32 * EPI + 128, 1)
         }
       }
     }
-    if (!ok) {
-      raise_abort();
-      const int first = it > S::STAGES ? it - S::STAGES : 0;
-      for (int j = first; j < it; ++j)
-        mbar_wait_bounded(full_bar(j % S::STAGES), (j / S::STAGES) & 1, nullptr, kL1DrainNs);
-    }
+    if (!ok) raise_abort();
+    // no exit with a copy in flight, also where only another role gave up
+    const int first = it > S::STAGES ? it - S::STAGES : 0;
+    for (int j = first; j < it; ++j)
+      mbar_wait_bounded(full_bar(j % S::STAGES), (j / S::STAGES) & 1, nullptr, kL1DrainNs);
   } else if (warp == 1 && lane == 0) {
     // ---------------------------------------------------------- MMA issuer
     constexpr uint32_t idesc = mma_idesc(1u, S::BN, S::BM);

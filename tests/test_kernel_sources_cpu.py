@@ -48,3 +48,20 @@ def test_pair_allocations_follow_a_cluster_barrier():
             assert "cluster_sync_all()" in before or (
                 0 <= before.find("cluster_arrive_relaxed()") < before.find("cluster_wait()")), name
     assert found >= 2
+
+
+def test_no_cta_leaves_with_copies_in_flight():
+    """A producer that has issued its last copy may leave while another role
+    gives up waiting for it, so the wait for the copies in flight depends on no
+    outcome: each single-CTA kernel that loads tiles ends its producer with one,
+    outside of any `if (!ok) { ... }`."""
+    found = 0
+    for name, text in _sources("*.cu").items():
+        for kernel in re.split(r"__global__", text)[1:]:
+            if "tma_load_2d(" not in kernel:
+                continue
+            found += 1
+            assert re.search(r"mbar_wait_bounded\(full_bar\([^;]*nullptr, k\w+Ns\)", kernel), name
+            for block in re.findall(r"if \(!ok\) \{([^{}]*)\}", kernel):
+                assert "full_bar(" not in block, name
+    assert found >= 6
