@@ -55,8 +55,10 @@ typedef enum {
 
 typedef enum {
   DDF_FP32 = 0,      /* FP32 (no TF32): widths that are multiples of 256 on the tensor cores,
-                        each operand split exactly into three bf16 values, others on CUDA
-                        cores */
+                        each operand split exactly into three bf16 values and six of the
+                        nine products summed (those left out are at most 2^-25 of the
+                        product each), others on CUDA cores; infinities carry through
+                        either way */
   DDF_BF16 = 1,      /* bf16 operands, FP32 accumulation on tcgen05 tensor cores */
   DDF_FP8_E4M3 = 2   /* e4m3 operands (layers 2..H), FP32 accumulation on tcgen05 */
 } ddf_precision;

@@ -4,8 +4,11 @@
 // which is exact for normal numbers (3 x 8 significand bits; every remainder
 // is a float32 subtraction without rounding), and summing the six products
 //   a2 w0 + a0 w2 + a1 w1 + a1 w0 + a0 w1 + a0 w0
-// of bf16 operands, each exact in FP32. The three products left out are below
-// 2^-26 of |a w| each, and of random sign (the pieces are rounded to nearest).
+// of bf16 operands, each exact in FP32. Of the three products left out a1 w2 and
+// a2 w1 reach 2^-25 of |a w| (|x1| <= 2^-8 |x|, |x2| <= 2^-17 |x|), a2 w2 2^-34, all
+// of random sign (the pieces are rounded to nearest). An infinite activation
+// meets each weight once, in a2 w0, and gives what an FP32 FMA gives (unless the
+// weight is so small, under 2^-133, that its first piece is 0).
 //
 // What bounds it: the tensor pipe, at six bf16 MMAs per FP32 one, and between
 // two tiles the outputs (the epilogue warps hold a tile's sums in registers, so
@@ -91,6 +94,43 @@ __device__ __forceinline__ F32Tile f32_tile(const F32Plan& f, int t, int num_n) 
   return F32Tile{m * 256, (t - m * num_n) * 256 + sub * n, n};
 }
 
+// The pieces of COLS outputs (>= 0, no NaN), as f32_split gives them, 16 at a time,
+// plane by plane and packed in pairs. An infinity's pieces come out as bf16's
+// largest value, infinity and NaN, which the sum of all third pieces shows; they
+// are then looked for and stored again. With the selects of f32_split for each
+// output the drain has too few registers (16,387 rays 1,471 us without a rule for
+// infinities, 1,503 with the selects, 1,474 so).
+template <int COLS>
+__device__ __forceinline__ void f32_store_planes(float* x, __nv_bfloat16* dst, size_t plane) {
+  const __nv_bfloat162 most = __halves2bfloat162(__ushort_as_bfloat16(0x7f7f),
+                                                 __ushort_as_bfloat16(0x7f7f));
+  __nv_bfloat162 sum = __halves2bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0));
+#pragma unroll
+  for (int c = 0; c < COLS; c += 16) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      uint32_t w[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float &a = x[c + 2 * i], &b = x[c + 2 * i + 1];
+        __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+        if (j == 0) v = __hmin2(v, most);
+        if (j == 2) sum = __hadd2(sum, v);
+        w[i] = *reinterpret_cast<const uint32_t*>(&v);
+        a -= __uint_as_float(w[i] << 16);
+        b -= __uint_as_float(w[i] & 0xffff0000u);
+      }
+      st_global_256(dst + j * plane + c, w);
+    }
+  }
+  if (__builtin_expect(__hbeq2(sum, sum), 1)) return;
+  for (int i = 0; i < COLS; ++i) {
+    if (!__hisnan(dst[2 * plane + i])) continue;
+    dst[i] = dst[plane + i] = __ushort_as_bfloat16(0);
+    dst[2 * plane + i] = __ushort_as_bfloat16(0x7f80);
+  }
+}
+
 // One warp's part of a tile: COLS columns of its 32 rows, the accumulators of
 // every 32 of K added up (`it` counts them), then bias, ReLU and the output at the
 // row and column `where` gives (asked late: its registers are not there before).
@@ -141,18 +181,8 @@ __device__ __forceinline__ bool f32_drain(const TcF32Params& p, uint32_t trow, i
       st_global_256(dst + 8 * c, w);
     }
   } else {  // the next layer's operand: three bf16 planes
-#pragma unroll
-    for (int c = 0; c < COLS / 16; ++c) {
-      uint4 lo[3], hi[3];
-      f32_split8(acc + 16 * c, lo);
-      f32_split8(acc + 16 * c + 8, hi);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const uint32_t w[8] = {lo[j].x, lo[j].y, lo[j].z, lo[j].w,
-                               hi[j].x, hi[j].y, hi[j].z, hi[j].w};
-        st_global_256(p.out_planes + (static_cast<size_t>(j) * p.M + row) * p.N + n0 + 16 * c, w);
-      }
-    }
+    f32_store_planes<COLS>(acc, p.out_planes + static_cast<size_t>(row) * p.N + n0,
+                           static_cast<size_t>(p.M) * p.N);
   }
   return true;
 }
