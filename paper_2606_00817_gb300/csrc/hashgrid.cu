@@ -771,16 +771,18 @@ __global__ void hg_pack_image_kernel(const float* __restrict__ w, int K, uint8_t
 
 int hashgrid_smem_bytes(int H) { return HgSmem::bytes(H); }
 
+constexpr int kHgMaxLayers = 4;
 constexpr int kHgCtasPerSm = 4;  // __launch_bounds__(128, 4): 128 registers per thread
 
 // Shared memory for the tensor-core kernel: its dynamic size, and a carveout
 // just large enough for kHgCtasPerSm CTAs, so that the rest of the SM's
 // unified memory stays L1 cache for the table gathers (about a third of them
-// hit there).
+// hit there). The limits of the dynamic sizes, here and below, are constants: they
+// are the function's, and host threads with other fields set them too.
 cudaError_t hashgrid_tc_configure(int H) {
   cudaError_t e = cudaFuncSetAttribute(hashgrid_tc_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       HgSmem::bytes(H));
+                                       HgSmem::bytes(kHgMaxLayers));
   if (e != cudaSuccess) return e;
   int dev = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -829,14 +831,21 @@ int hashgrid_tc_blocks_per_sm(int H) {
   return n;
 }
 
+namespace {
+constexpr int hg_f32_bytes(int H) { return (hg_wt_floats(H) + kHgW * kHgF32Ld) * 4; }
+constexpr int hg_fwd_bytes(int H) { return (hg_wt_floats(H) + 2 * kHgW * kHgLda) * 4; }
+constexpr int hg_bwd_bytes(int H) { return (hg_bwd_floats(H) + 2 * kHgW * kHgLda) * 4; }
+}  // namespace
+
 cudaError_t launch_hashgrid_f32(const HashGridParams& g, const float2* table, const float* mlp,
                                 int H, RaySoA rays, int64_t M, HeadOut out, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
   if (H < 1 || H > 4 || (reinterpret_cast<uintptr_t>(table) & 15u) != 0)
     return cudaErrorInvalidValue;
-  const int smem = (hg_wt_floats(H) + kHgW * kHgF32Ld) * static_cast<int>(sizeof(float));
-  cudaError_t e = cudaFuncSetAttribute(hashgrid_f32_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int smem = hg_f32_bytes(H);
+  cudaError_t e =
+      cudaFuncSetAttribute(hashgrid_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           hg_f32_bytes(kHgMaxLayers));
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -855,9 +864,10 @@ cudaError_t launch_hg_train_fwd(const HashGridParams& g, const float2* table, co
   if (B <= 0) return cudaSuccess;
   if (H < 1 || H > 4 || (reinterpret_cast<uintptr_t>(table) & 15u) != 0)
     return cudaErrorInvalidValue;
-  const int smem = (hg_wt_floats(H) + 2 * kHgW * kHgLda) * static_cast<int>(sizeof(float));
-  cudaError_t e = cudaFuncSetAttribute(hg_train_fwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int smem = hg_fwd_bytes(H);
+  cudaError_t e =
+      cudaFuncSetAttribute(hg_train_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           hg_fwd_bytes(kHgMaxLayers));
   if (e != cudaSuccess) return e;
   const int64_t blocks = (B + kHgTrainRays - 1) / kHgTrainRays;
   hg_train_fwd_kernel<<<static_cast<unsigned>(blocks), kHgTrainThreads, smem, s>>>(
@@ -871,9 +881,10 @@ cudaError_t launch_hg_train_bwd(const HashGridParams& g, const float* mlp, int H
   if (B <= 0) return cudaSuccess;
   if (H < 1 || H > 4) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(grad_table) & 7u) != 0) return cudaErrorInvalidValue;
-  const int smem = (hg_bwd_floats(H) + 2 * kHgW * kHgLda) * static_cast<int>(sizeof(float));
-  cudaError_t e = cudaFuncSetAttribute(hg_train_bwd_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int smem = hg_bwd_bytes(H);
+  cudaError_t e =
+      cudaFuncSetAttribute(hg_train_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           hg_bwd_bytes(kHgMaxLayers));
   if (e != cudaSuccess) return e;
   const int64_t blocks = (B + kHgTrainRays - 1) / kHgTrainRays;
   hg_train_bwd_kernel<<<static_cast<unsigned>(blocks), kHgTrainThreads, smem, s>>>(

@@ -61,6 +61,8 @@ __device__ __forceinline__ void store_row8(F32Planes* out, int64_t at, int64_t p
 }
 
 constexpr int kEncRays = 64;  // rays per block of the encoder
+constexpr int kEncMaxLd = 200;  // 16 bands, rounded up to 8
+constexpr int enc_bytes(int ld) { return kEncRays * (ld + 1) * 4; }
 
 // One block encodes kEncRays rays: each thread builds its ray's row in shared
 // memory (row stride ld+1 to spread banks), then the block writes the rows,
@@ -111,12 +113,12 @@ template <typename T>
 cudaError_t launch_encode(RaySoA rays, int64_t M, int L, int ld, T* out, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
   const int64_t blocks = (M + kEncRays - 1) / kEncRays;
-  const size_t smem = static_cast<size_t>(kEncRays) * (ld + 1) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(encode_kernel<T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  if (ld > kEncMaxLd) return cudaErrorInvalidValue;
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(
+      encode_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc_bytes(kEncMaxLd));
   if (e != cudaSuccess) return e;
-  encode_kernel<T><<<static_cast<unsigned>(blocks), kEncRays, smem, s>>>(rays, M, L, ld, out);
+  encode_kernel<T><<<static_cast<unsigned>(blocks), kEncRays, enc_bytes(ld), s>>>(rays, M, L, ld, out);
   return cudaGetLastError();
 }
 

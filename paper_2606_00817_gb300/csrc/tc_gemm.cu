@@ -268,11 +268,14 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const TcG
                        int grid, cudaStream_t s) {
   using S = TcShape<BN, IN_FP8>;
   auto kern = tc_gemm_kernel<BN, IN_FP8, OUT_FP8, EPI>;
-  // applies to the current device; cheap enough to repeat on every launch
   if (p.k_splits > 1 && (p.K + S::BK - 1) / S::BK < p.k_splits) return cudaErrorInvalidValue;
   if (p.mn_major && IN_FP8) return cudaErrorInvalidValue;
+  if (p.N > kMaxStagedColumns) return cudaErrorInvalidValue;
   const int smem = S::SMEM_BYTES + epi_vector_bytes(p.N);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // applies to the current device; cheap enough to repeat on every launch, and a
+  // constant: the limit is the function's, and host threads with other fields set it too
+  constexpr int kLimit = S::SMEM_BYTES + epi_vector_bytes(kMaxStagedColumns);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLimit);
   if (e != cudaSuccess) return e;
   kern<<<grid, 64 + 32 * EPI, smem, s>>>(tmA, tmB, p);
   return cudaGetLastError();

@@ -360,8 +360,11 @@ cudaError_t launch_pair_one(const CUtensorMap& tmA, const CUtensorMap& tmB, cons
                             const TcGemmParams& p, int grid, cudaStream_t s) {
   using S = PairShape<IN_FP8, STAGED, EPI>;
   auto kern = tc_gemm_pair_kernel<IN_FP8, OUT_FP8, STAGED, TM, EPI>;
+  if (p.N > kMaxStagedColumns) return cudaErrorInvalidValue;
   const int smem = S::smem_bytes(p.N);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       S::smem_bytes(kMaxStagedColumns));
   if (e != cudaSuccess) return e;
   kern<<<grid, S::THREADS, smem, s>>>(tmA, tmB, tmO, p);
   return cudaGetLastError();
@@ -372,7 +375,8 @@ int max_pairs_for() {
   using S = PairShape<IN_FP8, STAGED, EPI>;
   auto kern = tc_gemm_pair_kernel<IN_FP8, false, STAGED, 0, EPI>;
   const int smem = S::smem_bytes(kMaxStagedColumns);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           S::smem_bytes(kMaxStagedColumns)) != cudaSuccess)
     return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2, 1, 1);

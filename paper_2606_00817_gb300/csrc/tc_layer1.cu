@@ -300,7 +300,9 @@ cudaError_t launch_l1(const CUtensorMap& tmB, const CUtensorMap& tmO, RaySoA ray
                       const TcGemmParams& p, int grid, cudaStream_t s) {
   auto kern = tc_layer1_kernel<OUT_FP8, EPI>;
   const int smem = L1Shape<EPI>::smem_bytes(p.N);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       L1Shape<EPI>::smem_bytes(kMaxStagedColumns));
   if (e != cudaSuccess) return e;
   kern<<<grid, 64 + 32 * EPI + 128, smem, s>>>(tmB, tmO, rays, L, p);
   return cudaGetLastError();

@@ -43,6 +43,7 @@ constexpr int kNwSlots = 16;      // most chunks a ring holds
 constexpr int kNwBlock = 16384;   // 128 rows x 64 K of a tile
 constexpr int kNwCtrl = 512;
 constexpr int kNwSmemMax = 227 * 1024 - 1024;  // less the base alignment
+constexpr int kNwSmemLimit = 227 * 1024;
 
 // Byte offset of element pair (even column c) of row r in the operand tile.
 __device__ __forceinline__ uint32_t nw_off(int r, int c) {
@@ -362,8 +363,9 @@ __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
 template <int W>
 cudaError_t launch_w(const NarrowMaps& maps, const NarrowParams& p, const NwShape& s,
                      const RaySoA& rays, const HeadOut& out, int num_sms, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(tc_narrow_kernel<W>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(
+      tc_narrow_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNwSmemLimit);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (p.M + 127) / 128;
   const int grid = static_cast<int>(tiles < num_sms ? tiles : num_sms);

@@ -238,6 +238,11 @@ small_encode_kernel(const __grid_constant__ RaySoA rays, int64_t M, int L, int l
 // columns one chain of FMAs in column order, then the blocks in order, as the
 // default tiles and finish_heads_kernel add them.
 constexpr int kSmHeadRays = 8;
+__host__ __device__ constexpr int sm_heads_bytes(int nb, int blk) {
+  return ((2 + kSmHeadRays) * nb * (blk + 1) + kSmHeadRays * nb * 2) * 4;
+}
+// of the widest field, in blocks of 128
+constexpr int kSmHeadsLimit = sm_heads_bytes(kMaxStagedColumns / 128, 128);
 
 __global__ void __launch_bounds__(256)
 small_heads_kernel(const float* __restrict__ X, int M, int W, int blk,
@@ -339,9 +344,11 @@ cudaError_t launch_small_heads(const float* X, int M, int W, int blk, const floa
   if (M <= 0) return cudaSuccess;
   if (W % blk != 0 || blk % 4 != 0) return cudaErrorInvalidValue;
   const int nb = W / blk;
-  const int smem = ((2 + kSmHeadRays) * nb * (blk + 1) + kSmHeadRays * nb * 2) * 4;
-  cudaError_t e = cudaFuncSetAttribute(small_heads_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int smem = sm_heads_bytes(nb, blk);
+  if (smem > kSmHeadsLimit) return cudaErrorInvalidValue;
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(
+      small_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmHeadsLimit);
   if (e != cudaSuccess) return e;
   return launch_dependent<const float*, int, int, int, const float*, const float*, HeadOut>(
       small_heads_kernel, (M + kSmHeadRays - 1) / kSmHeadRays, 256, smem, s, X, M, W, blk, wo, bo,

@@ -47,7 +47,8 @@ constexpr int kTrThreads = 256 + 32;  // 8 compute warps, the producer
 constexpr int kTrBlock = 16384;       // 128 rows x 64 K: a K block of the tile, and a weight chunk
 constexpr int kTrSlots = 8;           // most ring slots
 constexpr int kTrCtrl = 512;
-constexpr int kTrSmemMax = 227 * 1024 - 1024;
+constexpr int kTrSmemMax = 227 * 1024 - 1024;  // less the base alignment
+constexpr int kTrSmemLimit = 227 * 1024;
 
 struct TrShape {
   int kb1;    // K blocks of the encoding
@@ -490,8 +491,9 @@ __global__ void __launch_bounds__(kTrThreads, 1)
 
 template <int C>
 cudaError_t configure(const TrShape& s, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
-  cudaError_t e = cudaFuncSetAttribute(tc_trace_kernel<C>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+  // a constant: the limit is the function's, and host threads with other fields set it too
+  cudaError_t e = cudaFuncSetAttribute(
+      tc_trace_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrSmemLimit);
   if (e != cudaSuccess) return e;
   *cfg = cudaLaunchConfig_t{};
   cfg->blockDim = dim3(kTrThreads);

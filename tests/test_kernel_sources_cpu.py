@@ -65,3 +65,19 @@ def test_no_cta_leaves_with_copies_in_flight():
             for block in re.findall(r"if \(!ok\) \{([^{}]*)\}", kernel):
                 assert "full_bar(" not in block, name
     assert found >= 6
+
+
+def test_shared_memory_limits_are_constants():
+    """A kernel's limit of dynamic shared memory belongs to the function, not to a
+    field or a host thread: a launcher that set it to its own field's size could
+    lower it between another thread's setting and launch. Every limit is made of
+    constants only."""
+    found = 0
+    constant = re.compile(r"k[A-Z]\w*|[A-Z][A-Z0-9_]*|[A-Z]\w*Shape|HgSmem|\w*bytes|\d+")
+    for name, text in _sources("*.cu").items():
+        for limit in re.findall(r"cudaFuncAttributeMaxDynamicSharedMemorySize,\s*(.*?)\)\s*(?:;|!=|==)",
+                                text, flags=re.S):
+            found += 1
+            for word in re.findall(r"\w+", limit):
+                assert constant.fullmatch(word), (name, limit)
+    assert found >= 15
