@@ -1848,6 +1848,14 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   if (ws == nullptr || ddf_internal_workspace_bytes(h, n) > ws_bytes)
     return fail(DDF_ERR_INVALID_ARG, "workspace too small for this batch");
   DeviceGuard g(h->cfg.device);
+  if (!h->sizes_loaded && h->tile_auto && !h->tmSmall.empty()) {
+    // a batch of another size may come in a frame, or while a stream is captured;
+    // other fields have the same kernels for every size
+    const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
+    DDF_CK(ddf::load_small_kernels(fp8));
+    DDF_CK(ddf::load_step_query_kernels(fp8));
+    h->sizes_loaded = true;
+  }
   const int W = h->cfg.width;
   const bool f32 = h->cfg.precision == DDF_FP32;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };

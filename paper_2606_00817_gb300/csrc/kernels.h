@@ -292,6 +292,16 @@ cudaError_t launch_small_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA
                                const CUtensorMap& tmB, const TcGemmParams& p, cudaStream_t s);
 cudaError_t launch_small_encode(const RaySoA& rays, int64_t M, int L, int ld, __nv_bfloat16* out,
                                 cudaStream_t s);
+// Loads the kernels of queries by tc_small.cu and by tc_steps.cu, which CUDA
+// otherwise does at each one's first launch.
+cudaError_t load_small_kernels(bool fp8);
+cudaError_t load_step_query_kernels(bool fp8);
+inline cudaError_t load_kernels(const void* const* kernels, int n) {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaFuncGetAttributes(&a, kernels[i]);
+  return e;
+}
 cudaError_t launch_small_heads(const float* X, int M, int W, int blk, const float* wo,
                                const float* bo, const HeadOut& o, cudaStream_t s);
 // The heads after launch_step_layer's last layer: out_f32 as X, the same tiles.

@@ -82,7 +82,8 @@ ddf_status scratch_address(int dev, void** out) {
 //    field, about 49,300 for 78->128x4), else DDF_ERR_INVALID_ARG names the
 //    limit. Hash-grid fields need no scratch, so their batches have no limit.
 //  * The first call on a device looks up the scratch address (and loads the
-//    module there); make that first call before any stream capture.
+//    module there), and the first call of a handle loads the kernels of every
+//    batch size; make that first call before any stream capture.
 //  * Every call, from every handle, shares the one array and leaves its
 //    contents behind. Nothing in it has to start at zero: each call writes
 //    every scratch byte it reads before reading it. Calls that overlap on the

@@ -315,6 +315,20 @@ cudaError_t launch_layer(const CUtensorMap& tmA, const CUtensorMap& tmB, const T
 
 }  // namespace
 
+cudaError_t load_small_kernels(bool fp8) {
+  // e4m3: the first layer, the others, the last one, a single one
+  const void* bf16[] = {(const void*)tc_small_kernel<false, kOutBf16>,
+                        (const void*)tc_small_kernel<false, kOutF32>};
+  const void* e4m3[] = {(const void*)tc_small_kernel<false, kOutFp8>,
+                        (const void*)tc_small_kernel<true, kOutFp8>,
+                        (const void*)tc_small_kernel<true, kOutF32>,
+                        (const void*)tc_small_kernel<false, kOutF32>};
+  const void* both[] = {(const void*)small_encode_kernel, (const void*)small_heads_kernel};
+  cudaError_t e = load_kernels(both, 2);
+  if (e == cudaSuccess) e = fp8 ? load_kernels(e4m3, 4) : load_kernels(bf16, 2);
+  return e;
+}
+
 cudaError_t launch_small_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
                                const CUtensorMap& tmB, const TcGemmParams& p, cudaStream_t s) {
   if (p.M <= 0) return cudaSuccess;

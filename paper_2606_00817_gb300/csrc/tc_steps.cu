@@ -531,6 +531,19 @@ cudaError_t launch_layer(const CUtensorMap& tmA, const CUtensorMap& tmB, const C
 
 }  // namespace
 
+cudaError_t load_step_query_kernels(bool fp8) {
+  const void* bf16[] = {(const void*)tc_step_kernel<false, false, false>,
+                        (const void*)tc_step_kernel<false, false, true>};
+  const void* e4m3[] = {(const void*)tc_step_kernel<false, true, false>,
+                        (const void*)tc_step_kernel<true, true, false>,
+                        (const void*)tc_step_kernel<true, false, true>,
+                        (const void*)tc_step_kernel<false, false, true>};
+  const void* heads = (const void*)step_heads_kernel;
+  cudaError_t e = load_kernels(&heads, 1);
+  if (e == cudaSuccess) e = fp8 ? load_kernels(e4m3, 4) : load_kernels(bf16, 2);
+  return e;
+}
+
 cudaError_t launch_step_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
                               const CUtensorMap& tmB, const CUtensorMap& tmB64,
                               const TcGemmParams& p, const StepTiles& st, bool first,
