@@ -571,8 +571,10 @@ ddf_status ddf_get_tile(ddf_handle h, int32_t which, ddf_tile* tile);
  * over 3 rounds, one query each, and keep their best round (so a clock that
  * drifts under the power cap affects all alike): phase 1 times every launch
  * of the query, phase 2 the encoding and layer-1 launches only (CUDA events
- * around each launch). A bf16 field of width 128 or 256 keeps its one kernel
- * where none of the tiles is faster. ms_out (nullable,
+ * around each launch). Where a batch of this size takes other kernels as long
+ * as no tile is set (ddf_set_tile), whole queries by them and by the tiles just
+ * chosen are timed in turn, 3 times each, and if none of the tiles is faster the
+ * handle is left with no tile set. ms_out (nullable,
  * n_out >= 18) receives the per-query ms of phase 1 in [0..8] (7, 8 unused)
  * and of phase 2 in [9..17], -1 where a candidate was skipped or rejected.
  * Synchronous; allocates 16 n bytes of device memory while it runs. A no-op

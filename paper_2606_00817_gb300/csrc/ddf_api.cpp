@@ -1772,24 +1772,52 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
     result = ddf_set_tile(h, 0, &kCands[best_h]);
     if (result == DDF_OK) best_f = tune(0, kTileCands, true, p2);
   }
-  // a narrow field's one-kernel query, against the tiles just chosen
-  bool fused_wins = false;
-  if (result == DDF_OK && best_f >= 0 && h->narrow &&
-      (result = ddf_set_tile(h, 1, &kCands[best_f])) == DDF_OK) {
-    double layered = 1e30, fused = 1e30;
+  // the kernels this batch takes where no tile is set, against the tiles just
+  // chosen, unless they are among the candidates (from mid_rows on)
+  const ddf_tile plain{h->cfg.width % 256 == 0 ? 256 : 128, 4, 0, 0, 0};
+  const bool own = h->narrow || (!h->tmSmall.empty() &&
+                                 (h->tmBig.empty() ||
+                                  std::min<int64_t>(n, h->chunk) <
+                                      mid_rows(h->cfg.width, h->num_sms,
+                                               h->cfg.precision == DDF_FP8_E4M3)));
+  auto choose = [&](bool untuned) -> ddf_status {
+    ddf_status r = ddf_set_tile(h, 0, untuned ? &plain : &kCands[best_h]);
+    if (r == DDF_OK) r = ddf_set_tile(h, 1, untuned ? &plain : &kCands[best_f]);
+    h->tile_auto = r == DDF_OK && untuned;
+    return r;
+  };
+  // Device time of a whole query, launches of which may overlap: enqueued behind
+  // another one, so that the host is ahead.
+  auto whole = [&](double* ms) -> ddf_status {
+    ddf::HeadOut o{};
+    o.t = buf + 2 * n;
+    o.vis = o.t + n;
+    cudaEvent_t a = nullptr, b = nullptr;
+    ddf_status r = run_query(h, rays, n, o, st);
+    float t = 0.f;
+    cudaError_t e = cudaEventCreate(&a);
+    if (e == cudaSuccess) e = cudaEventCreate(&b);
+    if (e == cudaSuccess) e = cudaEventRecord(a, st);
+    if (r == DDF_OK && e == cudaSuccess) r = run_query(h, rays, n, o, st);
+    if (e == cudaSuccess) e = cudaEventRecord(b, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&t, a, b);
+    if (a != nullptr) cudaEventDestroy(a);
+    if (b != nullptr) cudaEventDestroy(b);
+    *ms = t;
+    return r != DDF_OK || e == cudaSuccess ? r : cuda_fail(e, "autotune: timing a query");
+  };
+  bool untuned_wins = false;
+  if (result == DDF_OK && best_f >= 0 && own && (result = choose(true)) == DDF_OK) {
+    double best[2] = {1e30, 1e30};
     bool pass = false;
-    h->tile_auto = true;
     result = check(&pass);
-    for (int round = 0; round < kRounds && result == DDF_OK && pass; ++round) {
-      double a = 0.0, b = 0.0;
-      if ((result = timed(false, &a)) != DDF_OK) break;
-      h->tile_auto = false;
-      if ((result = timed(false, &b)) != DDF_OK) break;
-      h->tile_auto = true;
-      fused = std::min(fused, a);
-      layered = std::min(layered, b);
+    for (int k = 0; k < 2 * kRounds && result == DDF_OK && pass; ++k) {
+      double t = 0.0;
+      if ((result = choose(k % 2 == 0)) == DDF_OK && (result = whole(&t)) == DDF_OK)
+        best[k % 2] = std::min(best[k % 2], t);
     }
-    fused_wins = pass && fused <= layered;
+    untuned_wins = pass && best[0] <= best[1];
   }
   for (int c = 0; ms_out != nullptr && c < kTileCands; ++c) {
     ms_out[c] = p1[c];
@@ -1803,10 +1831,7 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
     h->tile_auto = keep_auto;
     return result != DDF_OK ? result : fail(DDF_ERR_CUDA, "autotune: no candidate passed");
   }
-  ddf_status r = ddf_set_tile(h, 0, &kCands[best_h]);
-  if (r == DDF_OK) r = ddf_set_tile(h, 1, &kCands[best_f]);
-  h->tile_auto = r == DDF_OK && fused_wins;
-  return r;
+  return choose(untuned_wins);
 }
 
 }  // extern "C"
