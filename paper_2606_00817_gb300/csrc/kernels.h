@@ -50,7 +50,7 @@ struct TcGemmParams {
   int k_splits;
   size_t split_stride;     // elements between split outputs
   float* out_f32;
-  // 1-CTA kernel, nullable: device int holding the number of rows to compute
+  // tc_steps.cu only, nullable: device int holding the number of rows to compute
   // (at most M; M remains the row stride of the head partials)
   const int* m_dev;
   // 1-CTA kernel, bf16: both operands stored MN-major, A as [K x M] and B as
@@ -171,7 +171,7 @@ struct TcTile {
   int bn;
   int epi_warps;
   bool pair = false;    // 256 x 256 tile on a 2-CTA cluster (tc_gemm_pair.cu; bn 256, 4 warps)
-  bool staged = false;  // pair tile, or the fused layer-1 tile: outputs staged through shared memory
+  bool staged = false;  // pair or fused layer-1 tile: outputs staged through shared memory
   bool fused = false;   // layer 1 only: the encoding is built in shared memory (tc_layer1.cu)
 };
 
@@ -220,8 +220,9 @@ cudaError_t launch_sgemm_relu(const float* A, const float* W, const float* b, fl
 // FP32 layer on the tensor cores (tc_gemm_f32.cu): ReLU(A W^T + b) with both
 // operands given as three bf16 planes that add up to the FP32 values. tmA maps
 // A's planes as one [3 M x K] matrix, tmB W's as [3 N x K], with 128-row boxes, tmB32
-// the same with 32-row boxes; N % 256 == 0; clusters: as many as the GPU holds. The output is either the next layer's planes [3][M x N] or
-// FP32 rows [M x N], 32-byte aligned; bias 16-byte aligned.
+// the same with 32-row boxes; N % 256 == 0; clusters: as many as the GPU holds. The
+// output is either the next layer's planes [3][M x N] or FP32 rows [M x N], 32-byte
+// aligned; bias 16-byte aligned.
 struct TcF32Params {
   int M, N, K;
   const float* bias;
@@ -305,8 +306,8 @@ inline cudaError_t load_kernels(const void* const* kernels, int n) {
 cudaError_t launch_small_heads(const float* X, int M, int W, int blk, const float* wo,
                                const float* bo, const HeadOut& o, cudaStream_t s);
 // The heads after launch_step_layer's last layer: out_f32 as X, the same tiles.
-cudaError_t launch_step_heads(const float2* part, const float* X, int M, const StepTiles& st, const float* wo, const float* bo,
-                              const HeadOut& o, cudaStream_t s);
+cudaError_t launch_step_heads(const float2* part, const float* X, int M, const StepTiles& st,
+                              const float* wo, const float* bo, const HeadOut& o, cudaStream_t s);
 // From per-N-block partial dot products [nblk x M] (tensor-core path).
 cudaError_t launch_finish_heads(const float2* part, int nblk, int M, const float* bo, HeadOut o,
                                 cudaStream_t s);

@@ -104,11 +104,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // rows this launch computes: p.M, or fewer when a device-side count
-  // (written by an earlier kernel of the stream) is given; p.M stays the row
-  // stride of the head partials
-  const int m_rows = p.m_dev != nullptr ? min(*p.m_dev, p.M) : p.M;
-  const int num_m = (m_rows + S::BM - 1) / S::BM;
+  const int num_m = (p.M + S::BM - 1) / S::BM;
   const int num_n = p.N / BN;
   const int num_kb = (p.K + S::BK - 1) / S::BK;
   // split-K (mode 3): tile = (split, m block, n block); split s covers the
@@ -235,7 +231,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       int split, m_blk, n_blk;
       decode(tile, split, m_blk, n_blk);
       const int row = m_blk * S::BM + r_local;
-      const bool row_ok = row < m_rows;
+      const bool row_ok = row < p.M;
       const int n0 = n_blk * BN;
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                              static_cast<uint32_t>(b * BN);
@@ -300,7 +296,7 @@ int tc_gemm_smem_bytes(int bn, bool in_fp8) {
 cudaError_t launch_tc_gemm(const TcTile& tile, bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
                            const CUtensorMap& tmB, const TcGemmParams& p, int grid,
                            cudaStream_t s) {
-  if (!epi_out_aligned(p, out_fp8)) return cudaErrorInvalidValue;
+  if (!epi_out_aligned(p, out_fp8) || p.m_dev != nullptr) return cudaErrorInvalidValue;
   if (tile.bn == 256 && tile.epi_warps == 4) return launch_bn<256, 4>(in_fp8, out_fp8, tmA, tmB, p, grid, s);
   if (tile.bn == 256 && tile.epi_warps == 8) return launch_bn<256, 8>(in_fp8, out_fp8, tmA, tmB, p, grid, s);
   if (tile.bn == 128 && tile.epi_warps == 4) return launch_bn<128, 4>(in_fp8, out_fp8, tmA, tmB, p, grid, s);

@@ -13,7 +13,7 @@
 // What bounds it: the tensor pipe, at six bf16 MMAs per FP32 one, and between
 // two tiles the outputs (the epilogue warps hold a tile's sums in registers, so
 // the MMAs run at most two accumulators ahead of them). Measured through the
-// 126 -> 1280 x 8 field: 16,387 rays 1.53 ms against 9.53 ms on FFMA
+// 126 -> 1280 x 8 field: 16,387 rays 1.50 ms against 9.53 ms on FFMA
 // (sgemm_relu_kernel), without any output stores 1.18, without operand loads or
 // without reading the accumulators no less; 140,000 rays 11.8 ms, 1 ray 0.24
 // against 1.40 ms; at 256 x 3, 5,000 rays 0.06 against 0.128 ms. It wins at every
@@ -253,7 +253,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kF32Threads, 1)
   // brings 128 rows of A and half of the tile's rows of W
   auto load_stage = [&](int s, const F32Tile& t, int kb, uint32_t bar) {
     const uint32_t a = smem_u32(smem + s * kF32Stage);
-    const int m0 = t.m0 + static_cast<int>(rank) * 128, n0 = t.n0 + static_cast<int>(rank) * (t.n / 2);
+    const int m0 = t.m0 + static_cast<int>(rank) * 128;
+    const int n0 = t.n0 + static_cast<int>(rank) * (t.n / 2);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       tma_load_2d_pair(a + j * kF32Plane, &tmA, kb * 64, j * p.M + m0, bar);

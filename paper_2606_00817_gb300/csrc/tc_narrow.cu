@@ -82,9 +82,9 @@ NwShape nw_shape(int L, int W, int H) {
 
 template <int W>
 __global__ void __launch_bounds__(2 * kNwGroup + 32, 1)
-    tc_narrow_kernel(const __grid_constant__ NarrowMaps maps, const __grid_constant__ NarrowParams p,
-                     const NwShape sh, const __grid_constant__ RaySoA rays,
-                     const __grid_constant__ HeadOut out) {
+    tc_narrow_kernel(const __grid_constant__ NarrowMaps maps,
+                     const __grid_constant__ NarrowParams p, const NwShape sh,
+                     const __grid_constant__ RaySoA rays, const __grid_constant__ HeadOut out) {
   constexpr int kChunk = W * 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &

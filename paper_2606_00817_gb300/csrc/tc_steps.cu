@@ -327,10 +327,12 @@ step_encode_kernel(const __grid_constant__ RaySoA rays, const float* __restrict_
 
 // The step's outcome per active ray: s = the head's sum, steps += 1; s < eps is a
 // hit; else t += s, and the ray stays active unless t > t_max or it has used
-// max_steps evaluations. On a fixed grid of 256-thread blocks; `small_tiles` decides where s comes from: the head partials
-// of the 128 x bn tiles, or chains over X here, a block of bn columns a thread.
+// max_steps evaluations. On a fixed grid of 256-thread blocks. The tile plan of the
+// count decides where s comes from: rows whose tiles were all whole add up the
+// head partials these left, the others run the chains of their split tiles here
+// over X, a block of bn columns a thread.
 constexpr int kStUpdThreads = 256;
-constexpr int kStUpdRays = 16;  // rays of a block at a time in the small case
+constexpr int kStUpdRays = 16;  // rays of a block at a time where tiles were split
 
 __global__ void __launch_bounds__(kStUpdThreads)
 step_update_kernel(const __grid_constant__ StepUpdate u) {
@@ -364,7 +366,8 @@ step_update_kernel(const __grid_constant__ StepUpdate u) {
   };
   const int nb = u.tiles.num_n, lg = u.tiles.lg_bn, bn = 1 << lg;
   const TilePlan plan = tile_plan(cnt, u.tiles);
-  const int whole = plan.lg_split == 0 ? cnt : min(cnt, plan.big / nb * 128);  // rows of partials only
+  // rows of partials only
+  const int whole = plan.lg_split == 0 ? cnt : min(cnt, plan.big / nb * 128);
   for (int j0 = blockIdx.x * kStUpdThreads; j0 < whole; j0 += gridDim.x * kStUpdThreads) {
     const int j = j0 + static_cast<int>(threadIdx.x);
     float s = hb;
@@ -512,7 +515,7 @@ cudaError_t launch_step_encode(const RaySoA& rays, const float* t, const int* id
   if (cap <= 0 || ld % 8 != 0) return cudaErrorInvalidValue;
   const int blocks = (cap + kStEncRays - 1) / kStEncRays;
   return launch_chained<RaySoA, const float*, const int*, const int*, int*, int, int, int,
-                        __nv_bfloat16*>(step_encode_kernel, first, blocks < 4 * sms ? blocks : 4 * sms,
+                        __nv_bfloat16*>(step_encode_kernel, first, std::min(blocks, 4 * sms),
                                         3 * kStEncRays, kStEncRays * (ld + 8) * 2, s, rays, t, idx,
                                         count, next_count, cap, L, ld, out);
 }
@@ -550,7 +553,8 @@ cudaError_t launch_step_layer(bool in_fp8, bool out_fp8, const CUtensorMap& tmA,
                               cudaStream_t s) {
   const bool last = p.mode == 1;
   if (p.M <= 0) return cudaSuccess;
-  if ((st.lg_bn != 7 && st.lg_bn != 8) || p.N != st.num_n << st.lg_bn || p.bias == nullptr || st.sms < 1 ||
+  if ((st.lg_bn != 7 && st.lg_bn != 8) || p.N != st.num_n << st.lg_bn || p.bias == nullptr ||
+      st.sms < 1 ||
       (last && (p.head_w == nullptr || p.head_part == nullptr ||
                 (p.out_f32 == nullptr && st.x_tiles > 0) || out_fp8 ||
                 reinterpret_cast<uintptr_t>(p.out_f32) % 32 != 0)) ||
