@@ -584,7 +584,9 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
 
 /* Kernel timing. When on, the library brackets every launch with CUDA events
  * on the launching stream, grouped by kernel class:
- *   0 encode, 1 hidden-layer GEMM (layers 2..H), 2 head/finish, 3 first-layer GEMM.
+ *   0 encode, 1 hidden-layer GEMM (layers 2..H), 2 head/finish, 3 first-layer GEMM;
+ * a query or a trace that is one kernel counts as class 1. The events keep
+ * launches that would otherwise overlap apart.
  * ddf_profile_read synchronises, then stores per class the summed device time
  * in milliseconds (ms[4]) and launch counts (launches[4]), and resets them. */
 ddf_status ddf_profile_enable(ddf_handle h, int32_t on);

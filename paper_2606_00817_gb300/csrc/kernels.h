@@ -77,7 +77,7 @@ cudaError_t launch_encode_points_bf16(const float* px, const float* py, const fl
 cudaError_t launch_trace_init(int n, int* idx, int* count, float* t, int* steps, uint8_t* hit,
                               cudaStream_t s);
 // A whole trace in one persistent kernel (tc_trace.cu): SDF fields of width 128
-// .. 512 (a multiple of 128), 1 .. kTraceLayers layers. maps: every layer's bf16
+// .. 512 (a multiple of 128), 2 .. kTraceLayers layers. maps: every layer's bf16
 // weights with boxes of 64 K x 128 rows; queue: one device int of scratch.
 // Results are those of the step-by-step kernels, bit for bit.
 constexpr int kTraceLayers = 16;

@@ -145,7 +145,8 @@ __global__ void sum_partials_kernel(const float* __restrict__ part, int n, float
 constexpr int kSumThreads = 256;
 
 // The n partial sums added in order by one thread, from shared memory: with a
-// dependent global load each, 256 of them took 6.7 us.
+// dependent global load each, 256 of them took 6.7 us. A hash grid's step, of some
+// 200 us; a layered field's, of 3 ms, keeps the plain sum above.
 __global__ void __launch_bounds__(kSumThreads)
 sum_partials_staged_kernel(const float* __restrict__ part, int n, float* __restrict__ out) {
   __shared__ float s[kSumThreads];
