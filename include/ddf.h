@@ -182,8 +182,8 @@ ddf_status ddf_query_shadow_host(ddf_handle h, const float* const rays[6], int64
  *    bf16, about 49,300 for 78->128x4); larger n returns DDF_ERR_INVALID_ARG
  *    with the limit in the message. Hash-grid fields run one fused kernel
  *    with no scratch, so their batches have no such limit.
- *  - The first call on a device looks up the scratch address there, and the
- *    first call of a handle loads the kernels that its batches of any size
+ *  - The first call on a device looks up the scratch address there, and a
+ *    handle's first call loads the kernels that its batches of any size
  *    take (those of another tile at the first call after ddf_set_tile or
  *    ddf_autotune); make it before any stream capture. The other queries load
  *    the kernels of a batch size at the first batch of that size.

@@ -1841,6 +1841,25 @@ ddf_status ddf_autotune(ddf_handle h, const float* const rays[6], int64_t n, voi
 // instead of the handle (used by the allocation-free entry point in
 // noalloc.cu). Not part of the public header.
 
+namespace {
+
+// Loads the kernels of every batch size for the handle's precision, once a
+// device (asking for them again would cost a new handle's first call 7 us).
+ddf_status load_size_kernels(ddf_s* h) {
+  constexpr int kDevices = 64;
+  static std::atomic<unsigned> loaded[kDevices] = {};  // bit 0: bf16, bit 1: e4m3
+  const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
+  const unsigned bit = fp8 ? 2u : 1u;
+  const int dev = h->cfg.device;
+  if (dev < kDevices && (loaded[dev].load(std::memory_order_relaxed) & bit) != 0) return DDF_OK;
+  DDF_CK(ddf::load_small_kernels(fp8));
+  DDF_CK(ddf::load_step_query_kernels(fp8));
+  if (dev < kDevices) loaded[dev].fetch_or(bit, std::memory_order_relaxed);
+  return DDF_OK;
+}
+
+}  // namespace
+
 size_t ddf_internal_workspace_bytes(ddf_handle h, int64_t rows) {
   if (h->cfg.kind == DDF_KIND_HASHGRID) return 0;  // one fused kernel, no scratch
   const int W = h->cfg.width;
@@ -1873,14 +1892,9 @@ ddf_status ddf_internal_query_in_workspace(ddf_handle h, const float* const rays
   if (ws == nullptr || ddf_internal_workspace_bytes(h, n) > ws_bytes)
     return fail(DDF_ERR_INVALID_ARG, "workspace too small for this batch");
   DeviceGuard g(h->cfg.device);
-  if (!h->sizes_loaded && h->tile_auto && !h->tmSmall.empty()) {
-    // a batch of another size may come in a frame, or while a stream is captured;
-    // other fields have the same kernels for every size
-    const bool fp8 = h->cfg.precision == DDF_FP8_E4M3;
-    DDF_CK(ddf::load_small_kernels(fp8));
-    DDF_CK(ddf::load_step_query_kernels(fp8));
-    h->sizes_loaded = true;
-  }
+  // a batch of another size may come in a frame, or while a stream is captured;
+  // other fields have the same kernels for every size
+  if (h->tile_auto && !h->tmSmall.empty() && (s = load_size_kernels(h)) != DDF_OK) return s;
   const int W = h->cfg.width;
   const bool f32 = h->cfg.precision == DDF_FP32;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };

@@ -90,7 +90,6 @@ struct ddf_s {
   float2* ws_part = nullptr;
   float* ws_x = nullptr;  // small batches: the last layer's FP32 activations (one of ws_act)
   int64_t ws_x_rows = 0;
-  bool sizes_loaded = false;  // the kernels of every batch size of the allocation-free query
 
   uint32_t* status_dev = nullptr;
 
